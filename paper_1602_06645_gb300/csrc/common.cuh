@@ -56,21 +56,6 @@ struct BrickSummary {
     uint32_t flags;
 };
 
-// Band flags of one voxel at local brick position (x, y, z).
-__host__ __device__ __forceinline__ uint32_t band_flags(bool observed, float f, float lo_thr, float hi_thr, int x,
-                                                        int y, int z) {
-    if (!observed) return 0u;
-    const uint32_t b = (f <= lo_thr ? 1u : 0u) | (f >= hi_thr ? 2u : 0u);
-    uint32_t m = b;
-    if (x == 0) m |= b << 2;
-    if (x == 7) m |= b << 4;
-    if (y == 0) m |= b << 6;
-    if (y == 7) m |= b << 8;
-    if (z == 0) m |= b << 10;
-    if (z == 7) m |= b << 12;
-    return m;
-}
-
 struct Counters {
     uint32_t n_geo;      // geometry work list length
     uint32_t n_vis;      // visible brick list length
