@@ -21,6 +21,7 @@ struct tsdf_volume {
     int32_t ngz_all, ncz_all, slab_z0, slab_z1, zoff_g, zoff_c;
     float s_g, s_c, origin[3], mu, sigma, band;
     int32_t max_weight, colour_mode, sample_mode, culling, free_space;
+    bool plain_f;  // every F is a number within PLAIN_F (see Scratch::err)
     cudaStream_t stream;
     tsdf_allocator alloc;
     int device;

@@ -128,7 +128,13 @@ struct Scratch {
     uint32_t* need;         // per visible brick: listed bricks among it and its + neighbours not yet updated
     unsigned long long* ready;  // ready queue of the fused frame: frame_tag << 32 | brick
     struct FuseSync* fsync;
+    // err[0]: the device error word.  err[1]: 1 when the last restore (tsdf_write)
+    // left an F that is not a number or beyond PLAIN_F in magnitude; the fusion
+    // itself makes none (an average of such values and t <= 1 stays within
+    // them).  The summaries' minima and maxima pass over a NaN, so what relies
+    // on them to tell every voxel's F needs err[1] = 0 (tsdf_volume::plain_f).
     uint32_t* err;
+    uint16_t* ray_map;    // per geometry brick, of the ray caster
     uint2* vox;           // colour voxels that passed the band gate this frame: x | y << 16, z
     uint32_t vox_cap;
 };
@@ -204,8 +210,10 @@ cudaError_t launch_from_linear_u8(uint8_t* brick, const uint8_t* lin, const int3
                                   cudaStream_t stream);
 cudaError_t launch_from_linear_u32(uint32_t* brick, const uint32_t* lin, const int32_t dims[3], int z0, int z1,
                                    cudaStream_t stream);
+// Sets *odd_f (zeroed first) to 1 if some voxel's F is no number within PLAIN_F.
 cudaError_t launch_recompute_summaries(const float* F, const uint8_t* W, BrickSummary* summ, const int32_t ng[3],
-                                       float band, cudaStream_t stream);
+                                       float band, uint32_t* odd_f, cudaStream_t stream);
+constexpr float PLAIN_F = 1e30f;
 constexpr float CELL_EPS = 1e-5f;  // bound on trilinear overshoot of the corner range
 
 // Geometry-only fusion of one frame into caller-owned linear x-fastest F / w
@@ -278,9 +286,13 @@ struct RayConst {
     int32_t width, height;
     uint32_t max_iter;  // bound on samples per ray (never reached for valid parameters)
 };
-cudaError_t launch_raycast(const RayConst& c, const float* F, const uint8_t* W, const uint32_t* C,
-                           const BrickSummary* summ, float* range, float* vertex, float* normal, uint32_t* rgbw,
+// The map of the bricks a ray may cross without sampling (see k_ray_map), from
+// their summaries; plain_f: see Scratch::err.
+cudaError_t launch_ray_map(const BrickSummary* summ, const int32_t nb[3], bool plain_f, uint16_t* map,
                            cudaStream_t stream);
+// Reads the map of the volume as it is (launch_ray_map after its last change).
+cudaError_t launch_raycast(const RayConst& c, const float* F, const uint8_t* W, const uint32_t* C, const uint16_t* map,
+                           float* range, float* vertex, float* normal, uint32_t* rgbw, cudaStream_t stream);
 
 // ------------------------------------------------------- camera tracking --
 // One pyramid level of one tracking step (see tsdf_track in tsdf.h).

@@ -95,7 +95,8 @@ constexpr int SUM_WARPS = 8;
 __global__ void __launch_bounds__(SUM_WARPS * 32) k_summaries(const float* __restrict__ F,
                                                               const uint8_t* __restrict__ W,
                                                               BrickSummary* __restrict__ summ, int nx, int ny, int nz,
-                                                              int nbx, int nby, uint32_t nbt, float band) {
+                                                              int nbx, int nby, uint32_t nbt, float band,
+                                                              uint32_t* __restrict__ odd_f) {
     const uint32_t b = blockIdx.x * SUM_WARPS + (threadIdx.x >> 5);
     if (b >= nbt) return;
     const int lane = threadIdx.x & 31;
@@ -112,6 +113,7 @@ __global__ void __launch_bounds__(SUM_WARPS * 32) k_summaries(const float* __res
     const float inf = __int_as_float(0x7f800000), qnan = __int_as_float(0x7fffffff);
     float mn = inf, mx = -inf, mn_xf = inf, mx_xf = -inf, mn_zf = inf, mx_zf = -inf;
     uint32_t wmn = 0xFFFFFFFFu;
+    bool odd = false;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         const bool in = by * BRICK + ly < ny && bz * BRICK + lz + 2 * j < nz;
@@ -122,6 +124,7 @@ __global__ void __launch_bounds__(SUM_WARPS * 32) k_summaries(const float* __res
             const bool vox = in && bx * BRICK + lx + i < nx;
             const uint32_t wi = (w[j] >> (8 * i)) & 0xFFu;
             wmn = min(wmn, vox ? wi : 0xFFFFFFFFu);
+            odd = odd || (vox && !(fabsf(fv[i]) <= PLAIN_F));
             const float v = vox && wi ? fv[i] : qnan;  // fminf / fmaxf pass over a NaN
             gmn = fminf(gmn, v);
             gmx = fmaxf(gmx, v);
@@ -142,6 +145,7 @@ __global__ void __launch_bounds__(SUM_WARPS * 32) k_summaries(const float* __res
     const uint32_t all = lohi(mn, mx), xf = lohi(mn_xf, mx_xf), zf = lohi(mn_zf, mx_zf);
     uint32_t flags = all | (lx == 0 ? xf << 2 : xf << 4) | (ly == 0 ? all << 6 : 0u) | (ly == 7 ? all << 8 : 0u) |
                      (lz == 0 ? zf << 10 : zf << 12);
+    if (__any_sync(0xffffffffu, odd) && lane == 0) *odd_f = 1u;
     flags = __reduce_or_sync(0xffffffffu, flags);
     wmn = __reduce_min_sync(0xffffffffu, wmn);
 #pragma unroll
@@ -182,12 +186,14 @@ cudaError_t launch_from_linear_u32(uint32_t* b, const uint32_t* l, const int32_t
 }
 
 cudaError_t launch_recompute_summaries(const float* F, const uint8_t* W, BrickSummary* summ, const int32_t ng[3],
-                                       float band, cudaStream_t stream) {
+                                       float band, uint32_t* odd_f, cudaStream_t stream) {
+    const cudaError_t e = cudaMemsetAsync(odd_f, 0, sizeof(uint32_t), stream);
+    if (e != cudaSuccess) return e;
     const int nbx = (ng[0] + BRICK - 1) / BRICK, nby = (ng[1] + BRICK - 1) / BRICK, nbz = (ng[2] + BRICK - 1) / BRICK;
     const int64_t nbt = (int64_t)nbx * nby * nbz;
     if (nbt > 0)
         k_summaries<<<(unsigned)((nbt + SUM_WARPS - 1) / SUM_WARPS), SUM_WARPS * 32, 0, stream>>>(
-            F, W, summ, ng[0], ng[1], ng[2], nbx, nby, (uint32_t)nbt, band);
+            F, W, summ, ng[0], ng[1], ng[2], nbx, nby, (uint32_t)nbt, band, odd_f);
     return cudaGetLastError();
 }
 

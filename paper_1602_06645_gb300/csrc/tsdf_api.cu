@@ -180,10 +180,12 @@ void frame_constants(const tsdf_volume* v, const float Kd[9], const float Kr[9],
 }
 
 tsdf_status check_device_error(tsdf_volume* v) {
-    uint32_t e = 0;
-    cudaError_t ce = cudaMemcpyAsync(&e, v->scr.err, sizeof e, cudaMemcpyDeviceToHost, v->stream);
+    uint32_t w[2] = {0, 0};
+    cudaError_t ce = cudaMemcpyAsync(w, v->scr.err, sizeof w, cudaMemcpyDeviceToHost, v->stream);
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(v->stream);
     if (ce != cudaSuccess) return cuda_fail(v, ce, "device status read");
+    v->plain_f = w[1] == 0u && std::isfinite(1.0f / v->mu);
+    const uint32_t e = w[0];
     if (e) {
         cudaMemsetAsync(v->scr.err, 0, sizeof(uint32_t), v->stream);
         if (e == ERR_WAIT_TIMEOUT)
@@ -494,6 +496,7 @@ tsdf_status tsdf_create_ex(const int32_t dims_geo[3], const int32_t dims_col[3],
     v->sample_mode = p.sample_mode;
     v->culling = p.culling ? 1 : 0;
     v->free_space = p.update_free_space ? 1 : 0;
+    v->plain_f = std::isfinite(1.0f / mu);
 
     cudaError_t e = cudaGetDevice(&v->device);
     int sms = 0;
@@ -534,7 +537,7 @@ tsdf_status tsdf_create_ex(const int32_t dims_geo[3], const int32_t dims_col[3],
 
     const int64_t nbt = (int64_t)v->nb[0] * v->nb[1] * v->nb[2];
     const int64_t ncbt = (int64_t)v->ncb[0] * v->ncb[1] * v->ncb[2];
-    const size_t need = (size_t)nbt * BRICK_VOX * 5 + (size_t)ncbt * BRICK_VOX * 4 + (size_t)nbt * (sizeof(BrickSummary) + 25) +
+    const size_t need = (size_t)nbt * BRICK_VOX * 5 + (size_t)ncbt * BRICK_VOX * 4 + (size_t)nbt * (sizeof(BrickSummary) + 27) +
                         (size_t)vox_capacity(nbt) * sizeof(uint2);
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && need > free_b) {
@@ -551,7 +554,8 @@ tsdf_status tsdf_create_ex(const int32_t dims_geo[3], const int32_t dims_col[3],
     v->scr.vis_list = (uint32_t*)dev_alloc(v, (size_t)nbt * sizeof(uint32_t));
     v->scr.col_list = (uint32_t*)dev_alloc(v, (size_t)nbt * sizeof(uint32_t));
     v->scr.col_act = (uint8_t*)dev_alloc(v, (size_t)nbt);
-    v->scr.err = (uint32_t*)dev_alloc(v, sizeof(uint32_t));
+    v->scr.err = (uint32_t*)dev_alloc(v, 2 * sizeof(uint32_t));
+    v->scr.ray_map = (uint16_t*)dev_alloc(v, (size_t)nbt * sizeof(uint16_t));
     // fused frame: per-brick state bytes and neighbour counts, the ready queue and its counters
     v->scr.bstate = (uint8_t*)dev_alloc(v, (size_t)nbt);
     v->scr.need = (uint32_t*)dev_alloc(v, (size_t)nbt * sizeof(uint32_t));
@@ -566,7 +570,7 @@ tsdf_status tsdf_create_ex(const int32_t dims_geo[3], const int32_t dims_col[3],
     }
     v->scr.vox = (uint2*)dev_alloc(v, (size_t)v->scr.vox_cap * sizeof(uint2));
     if (!v->vol.F || !v->vol.W || !v->vol.C || !v->vol.summ || !v->scr.ctr || !v->scr.geo_list || !v->scr.vis_list ||
-        !v->scr.col_list || !v->scr.col_act || !v->scr.err || !v->scr.vox || !v->scr.bstate || !v->scr.need || !v->scr.ready ||
+        !v->scr.col_list || !v->scr.col_act || !v->scr.err || !v->scr.ray_map || !v->scr.vox || !v->scr.bstate || !v->scr.need || !v->scr.ready ||
         !v->scr.fsync) {
         tsdf_destroy(v);
         return TSDF_ERR_OOM;
@@ -582,7 +586,7 @@ tsdf_status tsdf_create_ex(const int32_t dims_geo[3], const int32_t dims_col[3],
     if (e == cudaSuccess) e = cudaMemsetAsync(v->vol.W, 0, (size_t)nbt * BRICK_VOX, v->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(v->vol.C, 0, (size_t)ncbt * BRICK_VOX * sizeof(uint32_t), v->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(v->scr.ctr, 0, sizeof(Counters), v->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(v->scr.err, 0, sizeof(uint32_t), v->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(v->scr.err, 0, 2 * sizeof(uint32_t), v->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(v->scr.ready, 0, (size_t)nbt * sizeof(unsigned long long), v->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(v->scr.fsync, 0, sizeof(FuseSync), v->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(v->scr.col_act, 0, (size_t)nbt, v->stream);
@@ -808,11 +812,13 @@ tsdf_status tsdf_read(tsdf_volume* v, float* tsdf, uint8_t* w_geo, uint32_t* rgb
 tsdf_status tsdf_write(tsdf_volume* v, const float* tsdf, const uint8_t* w_geo, const uint32_t* rgbw) {
     if (!v) return TSDF_ERR_INVALID_ARG;
     v->chain_ok = false;
+    v->plain_f = false;  // until the summaries of the new F say so (check_device_error)
     tsdf_status s = write_volume<float>(v, v->vol.F, tsdf, v->ng, launch_from_linear_f32);
     if (s == TSDF_OK) s = write_volume<uint8_t>(v, v->vol.W, w_geo, v->ng, launch_from_linear_u8);
     if (s == TSDF_OK) s = write_volume<uint32_t>(v, v->vol.C, rgbw, v->nc, launch_from_linear_u32);
     if (s != TSDF_OK) return s;
-    cudaError_t e = launch_recompute_summaries(v->vol.F, v->vol.W, v->vol.summ, v->ng, v->band, v->stream);
+    cudaError_t e = launch_recompute_summaries(v->vol.F, v->vol.W, v->vol.summ, v->ng, v->band, v->scr.err + 1,
+                                               v->stream);
     if (e != cudaSuccess) return cuda_fail(v, e, "summaries");
     return check_device_error(v);
 }

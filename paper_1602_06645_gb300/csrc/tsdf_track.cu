@@ -105,6 +105,7 @@ extern "C" tsdf_status tsdf_track(tsdf_volume* v, const uint16_t* depth_mm, tsdf
     if (!pose || !partials || !records) return fail(v, TSDF_ERR_OOM, "track: step buffers");
     if (e == cudaSuccess) e = cudaMemcpyAsync(pose, T_init, 16 * sizeof(double), cudaMemcpyHostToDevice, v->stream);
     if (e == cudaSuccess) e = tsdf::launch_track_pyramid(d_depth, W, H, p.levels, dl, v->stream);
+    if (e == cudaSuccess) e = tsdf::launch_ray_map(v->vol.summ, v->nb, v->plain_f, v->scr.ray_map, v->stream);
     if (e != cudaSuccess) return cuda_fail(v, e, "track: pyramid");
 
     // world -> prediction camera, as the fusion's frame constants invert a pose
@@ -139,7 +140,7 @@ extern "C" tsdf_status tsdf_track(tsdf_volume* v, const uint16_t* depth_mm, tsdf
         tsdf::RayConst rc;
         const tsdf_status rs = raycast_constants(v, Kl, T_world_depth_prev, tsdf_image_size{w, h}, &rp, rc);
         if (rs != TSDF_OK) return rs;
-        e = tsdf::launch_raycast(rc, v->vol.F, v->vol.W, v->vol.C, v->vol.summ, nullptr, PVl[l], PNl[l], nullptr,
+        e = tsdf::launch_raycast(rc, v->vol.F, v->vol.W, v->vol.C, v->scr.ray_map, nullptr, PVl[l], PNl[l], nullptr,
                                  v->stream);
         if (e != cudaSuccess) return cuda_fail(v, e, "track: prediction");
         L.w = w;
