@@ -309,10 +309,11 @@ cudaError_t launch_track_pyramid(const uint16_t* depth, int W, int H, int levels
 // Vertex and normal maps of one level; Kinv4 = (1/fx, 1/fy, -cx/fx, -cy/fy).
 cudaError_t launch_track_maps(const float* d, int w, int h, const float Kinv4[4], float* V, float* N,
                               cudaStream_t stream);
-int track_blocks(int npx);       // blocks (and binary64 partial-sum rows) of one step's reduction
+size_t track_partial_doubles(int npx);  // binary64 partial sums of one step's reduction
 size_t track_record_doubles();   // doubles recorded per step: 29 sums, 16 pose, 6 xi, 1 solved flag
-// One Gauss-Newton step at the device pose (binary64 row-major 4x4, updated in place).
-cudaError_t launch_track_step(const TrackLevel& L, double* pose, double* partials, double* record,
+// One Gauss-Newton step at the device pose (binary64 row-major 4x4, updated in
+// place).  *finished is 0 before the first step and after each.
+cudaError_t launch_track_step(const TrackLevel& L, double* pose, double* partials, unsigned* finished, double* record,
                               cudaStream_t stream);
 
 // ------------------------------------------------- mesh and texture maps --

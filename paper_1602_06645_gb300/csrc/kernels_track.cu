@@ -95,13 +95,176 @@ __device__ __forceinline__ void rigid3(const float* R, const float* t, float x, 
     Z = fmaf(R[6], x, fmaf(R[7], y, fmaf(R[8], z, t[2])));
 }
 
+// What bounds a step is the binary64 pipe, which takes about 64 cycles per
+// warp instruction on each quarter of an SM whatever the number of active
+// lanes, so both parts are written for few binary64 instructions per warp:
+//  * terms: the products of two binary32 factors are exact in binary64, so
+//    one fused multiply-add per sum rounds as a product and a sum would;
+//    the count is an integer; the 28 sums of a warp's lanes are reduced by
+//    halves (each exchange halves the sums a lane holds: 31 additions instead
+//    of 5 per sum, 145), the warps' and blocks' sums with one lane per sum;
+//  * solve: by the last block to finish, one warp, a lane per row or matrix
+//    entry (one thread alone took 28 us per step).
+// One launch per step; its blocks start while the previous step finishes and
+// read their first pixels before waiting for that step's pose.
+// Measured per step: 27.6 us at 640x480, 19.2 at 320x240, 16.8 at 160x120
+// (about 17 us of each is the fixed chain of wait, reduction and solve);
+// separate kernels for the terms and a one-thread solve took 57 us on average
+// over a frame's 19 steps.
+constexpr int NSLOT = 32;  // the 29 sums, padded
+
+// Sums of a warp's lanes: on return lane l holds the sum of v[l].
+__device__ __forceinline__ double warp_sums(double (&v)[NSLOT], int lane) {
+#pragma unroll
+    for (int h = NSLOT / 2; h >= 1; h >>= 1) {
+        const bool up = (lane & h) != 0;
+#pragma unroll
+        for (int k = 0; k < h; ++k) {
+            const double give = up ? v[k] : v[k + h], keep = up ? v[k + h] : v[k];
+            v[k] = keep + __shfl_xor_sync(0xffffffffu, give, h);
+        }
+    }
+    return v[0];
+}
+
+// exp coefficients of a rotation by angle a: row 0 sin(a)/a, row 1
+// (1 - cos(a))/a^2, row 2 (a - sin(a))/a^3, as power series in a^2
+// ((-1)^k / (2k + 1 + row)!, exact to binary64 for a <= 1/2: the first term
+// left out is below 0.25^8 / 17!).
+__constant__ double c_exp_series[3][8] = {
+    {1.0, -1.0 / 6, 1.0 / 120, -1.0 / 5040, 1.0 / 362880, -1.0 / 39916800, 1.0 / 6227020800.0,
+     -1.0 / 1307674368000.0},
+    {1.0 / 2, -1.0 / 24, 1.0 / 720, -1.0 / 40320, 1.0 / 3628800, -1.0 / 479001600, 1.0 / 87178291200.0,
+     -1.0 / 20922789888000.0},
+    {1.0 / 6, -1.0 / 120, 1.0 / 5040, -1.0 / 362880, 1.0 / 39916800, -1.0 / 6227020800.0, 1.0 / 1307674368000.0,
+     -1.0 / 355687428096000.0}};
+
+struct SolveShared {
+    double s[NSLOT], L[6][6], xi[6], coef[3], R[9], V[9], pose[16];
+};
+
+// One warp: solves A xi = -g by Cholesky (binary64; lane i holds row i) from
+// the sums in S.s and applies T <- exp(xi^) T; a matrix that is not positive
+// definite leaves T as it is.  The step's sums (29), its starting pose (16),
+// its xi (6) and whether it was solved go to record.
+__device__ void icp_solve(SolveShared& S, double* __restrict__ pose, double* __restrict__ record, int lane) {
+    const unsigned full = 0xffffffffu;
+    if (lane < 16) S.pose[lane] = pose[lane];
+    __syncwarp();
+    if (lane < NSUM) record[lane] = S.s[lane];
+    if (lane < 16) record[NSUM + lane] = S.pose[lane];
+    const int row = min(lane, 5);
+    double a[6];  // the row's lower part, then its factor's
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+        const int lo = min(row, j), hi = max(row, j);
+        a[j] = S.s[lo * 6 - lo * (lo - 1) / 2 + hi - lo];  // the upper triangle, row by row
+    }
+    double z = -S.s[21 + row], inv = 1.0;
+    bool ok = true;
+    // a pivot that is not positive marks the step unsolved and is replaced by
+    // 1 so the remaining arithmetic stays finite (its result is not used)
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+        double v = __shfl_sync(full, a[j], j);
+        if (!(v > 0.0)) {
+            ok = false;
+            v = 1.0;
+        }
+        const double y = rsqrt(v);  // 1 / L_jj
+        if (lane == j) inv = y;
+        a[j] = a[j] * y;
+#pragma unroll
+        for (int q = j + 1; q < 6; ++q) a[q] = __fma_rn(-a[j], __shfl_sync(full, a[j], q), a[q]);
+    }
+    if (lane < 6) {
+#pragma unroll
+        for (int j = 0; j < 6; ++j) S.L[lane][j] = a[j];
+    }
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {  // L y = -g: lane j's z becomes y_j
+        const double y = z * inv, yj = __shfl_sync(full, y, j);
+        z = lane == j ? y : (lane > j ? __fma_rn(-a[j], yj, z) : z);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int j = 5; j >= 0; --j) {  // L^T xi = y
+        const double x = z * inv, xj = __shfl_sync(full, x, j);
+        z = lane == j ? x : (lane < j ? __fma_rn(-S.L[j][row], xj, z) : z);
+    }
+    if (lane < 6) S.xi[lane] = ok ? z : 0.0;
+    __syncwarp();
+    if (ok) {
+        // exp(xi^): Rodrigues rotation, V(phi) rho translation
+        const double p0 = S.xi[3], p1 = S.xi[4], p2 = S.xi[5];
+        const double a2 = __fma_rn(p0, p0, __fma_rn(p1, p1, p2 * p2));
+        if (a2 <= 0.25) {
+            const double* cs = c_exp_series[min(lane, 2)];
+            double v = cs[7];
+#pragma unroll
+            for (int k = 6; k >= 0; --k) v = __fma_rn(v, a2, cs[k]);
+            if (lane < 3) S.coef[lane] = v;
+        } else if (lane == 0) {
+            const double an = sqrt(a2);
+            S.coef[0] = sin(an) / an;
+            S.coef[1] = (1.0 - cos(an)) / a2;
+            S.coef[2] = (an - sin(an)) / (a2 * an);
+        }
+        __syncwarp();
+        if (lane < 9) {  // entry (i, j) of R = I + cA W + cB W^2 and V = I + cB W + cC W^2, W = phi^
+            const int i = lane / 3, j = lane % 3;
+            const double pi = S.xi[3 + i], pj = S.xi[3 + j], pk = S.xi[3 + (i == j ? (i + 1) % 3 : 3 - i - j)],
+                         pl = S.xi[3 + (i + 2) % 3];
+            const double w = i == j ? 0.0 : ((j - i + 3) % 3 == 1 ? -pk : pk);
+            const double w2 = i == j ? -__fma_rn(pk, pk, pl * pl) : pi * pj;
+            const double e = i == j ? 1.0 : 0.0;
+            S.R[lane] = e + __fma_rn(S.coef[0], w, S.coef[1] * w2);
+            S.V[lane] = e + __fma_rn(S.coef[1], w, S.coef[2] * w2);
+        }
+        __syncwarp();
+        if (lane < 12) {
+            const int i = lane >> 2, j = lane & 3;
+            double v = 0.0;
+            if (j == 3) {
+#pragma unroll
+                for (int q = 0; q < 3; ++q) v = __fma_rn(S.V[i * 3 + q], S.xi[q], v);
+            }
+#pragma unroll
+            for (int q = 0; q < 3; ++q) v = __fma_rn(S.R[i * 3 + q], S.pose[q * 4 + j], v);
+            pose[lane] = v;
+        }
+    }
+    if (lane < 6) record[NSUM + 16 + lane] = S.xi[lane];
+    if (lane == 0) record[NSUM + 22] = ok ? 1.0 : 0.0;
+}
+
 // Per pixel: p = R V + t, m = R N; the prediction pixel of Rp p + tp through
 // Kl (nearest, inside, Z > 0, with a predicted normal); the distance and
 // normal gates; r = (p - q) . nq and J = (nq, p x nq).  The pose of the step
 // is read from the device (binary64, rounded once to binary32 here).  Each
-// block writes its binary64 partial sums, threads combined in a fixed order.
-__global__ void __launch_bounds__(TRACK_THREADS) k_icp_terms(TrackLevel L, const double* __restrict__ pose,
-                                                             double* __restrict__ partials) {
+// block writes its binary64 partial sums, threads combined in a fixed order;
+// the last block to finish sums the blocks' in a fixed order, solves and
+// updates the pose, and resets the count of finished blocks.
+__global__ void __launch_bounds__(TRACK_THREADS) k_icp_step(TrackLevel L, double* __restrict__ pose,
+                                                            double* __restrict__ partials,
+                                                            unsigned* __restrict__ finished,
+                                                            double* __restrict__ record) {
+    constexpr int NW = TRACK_THREADS / 32;
+    __shared__ double red[NW][NSLOT];
+    __shared__ SolveShared S;
+    __shared__ bool last;
+    const int npx = L.w * L.h;
+    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    // the vertex and normal maps are older than the previous step: read
+    // before waiting for it
+    float vx = 0.0f, vy = 0.0f, vz = 0.0f, nx = 0.0f, ny = 0.0f, nz = 0.0f;
+    auto fetch = [&](int k) {
+        vx = L.V[3 * k], vy = L.V[3 * k + 1], vz = L.V[3 * k + 2];
+        nx = L.N[3 * k], ny = L.N[3 * k + 1], nz = L.N[3 * k + 2];
+    };
+    if (i < npx) fetch(i);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     float R[9], t[3];
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
@@ -109,18 +272,19 @@ __global__ void __launch_bounds__(TRACK_THREADS) k_icp_terms(TrackLevel L, const
         for (int k = 0; k < 3; ++k) R[r * 3 + k] = (float)pose[r * 4 + k];
         t[r] = (float)pose[r * 4 + 3];
     }
-    double acc[NSUM];
+    double acc[NSLOT];
 #pragma unroll
-    for (int k = 0; k < NSUM; ++k) acc[k] = 0.0;
-    const int npx = L.w * L.h;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < npx; i += gridDim.x * blockDim.x) {
-        const float vx = L.V[3 * i], vy = L.V[3 * i + 1], vz = L.V[3 * i + 2];
-        const float nx = L.N[3 * i], ny = L.N[3 * i + 1], nz = L.N[3 * i + 2];
-        if (vz == 0.0f || (nx == 0.0f && ny == 0.0f && nz == 0.0f)) continue;
+    for (int k = 0; k < NSLOT; ++k) acc[k] = 0.0;
+    unsigned pairs = 0;
+    for (; i < npx; i += gridDim.x * blockDim.x) {
+        const float v0 = vx, v1 = vy, v2 = vz, m0 = nx, m1 = ny, m2 = nz;
+        const int next = i + gridDim.x * blockDim.x;
+        if (next < npx) fetch(next);
+        if (v2 == 0.0f || (m0 == 0.0f && m1 == 0.0f && m2 == 0.0f)) continue;
         float p[3], m[3], qc[3];
-        rigid3(R, t, vx, vy, vz, p[0], p[1], p[2]);
+        rigid3(R, t, v0, v1, v2, p[0], p[1], p[2]);
         const float zero[3] = {0.0f, 0.0f, 0.0f};
-        rigid3(R, zero, nx, ny, nz, m[0], m[1], m[2]);
+        rigid3(R, zero, m0, m1, m2, m[0], m[1], m[2]);
         rigid3(L.Rp, L.tp, p[0], p[1], p[2], qc[0], qc[1], qc[2]);
         if (!(qc[2] > 0.0f)) continue;
         const float rz = __frcp_rn(qc[2]);
@@ -136,158 +300,49 @@ __global__ void __launch_bounds__(TRACK_THREADS) k_icp_terms(TrackLevel L, const
         if (fmaf(e0, e0, fmaf(e1, e1, e2 * e2)) > L.max_dist2) continue;
         if (!(fmaf(m[0], n0, fmaf(m[1], n1, m[2] * n2)) >= L.min_cos)) continue;
         const float r = fmaf(e0, n0, fmaf(e1, n1, e2 * n2));
-        const double J[6] = {n0, n1, n2, (double)(p[1] * n2 - p[2] * n1), (double)(p[2] * n0 - p[0] * n2),
-                             (double)(p[0] * n1 - p[1] * n0)};
+        // J and r; the products of two of them are exact in binary64
+        const double J[7] = {n0, n1, n2, (double)(p[1] * n2 - p[2] * n1), (double)(p[2] * n0 - p[0] * n2),
+                             (double)(p[0] * n1 - p[1] * n0), (double)r};
         int k = 0;
 #pragma unroll
         for (int a = 0; a < 6; ++a)
 #pragma unroll
-            for (int b = a; b < 6; ++b) acc[k++] += J[a] * J[b];
+            for (int b = a; b < 6; ++b, ++k) acc[k] = __fma_rn(J[a], J[b], acc[k]);
 #pragma unroll
-        for (int a = 0; a < 6; ++a) acc[21 + a] += J[a] * (double)r;
-        acc[27] += (double)r * (double)r;
-        acc[28] += 1.0;
+        for (int a = 0; a < 7; ++a) acc[21 + a] = __fma_rn(J[a], J[6], acc[21 + a]);
+        ++pairs;
     }
-    // block: warp shuffles (fixed pattern), then warps in order
-    __shared__ double red[TRACK_THREADS / 32][NSUM];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    pairs = __reduce_add_sync(0xffffffffu, pairs);
+    const double sum = warp_sums(acc, lane);
+    red[warp][lane] = lane == 28 ? (double)pairs : sum;
+    __syncthreads();
+    if (warp == 0) {
+        double v = 0.0;
 #pragma unroll
-    for (int k = 0; k < NSUM; ++k) {
-        double v = acc[k];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) red[warp][k] = v;
+        for (int w = 0; w < NW; ++w) v += red[w][lane];
+        partials[(size_t)blockIdx.x * NSLOT + lane] = v;
+        __threadfence();
+        __syncwarp();
+        if (lane == 0) last = atomicAdd(finished, 1u) == gridDim.x - 1;
     }
     __syncthreads();
-    if (threadIdx.x < NSUM) {
-        double v = 0.0;
-        for (int w = 0; w < TRACK_THREADS / 32; ++w) v += red[w][threadIdx.x];
-        partials[(size_t)blockIdx.x * NSUM + threadIdx.x] = v;
-    }
-}
-
-// ------------------------------------------------------ solve and update --
-// One block of eight warps: the blocks' partials summed per sum in a fixed order,
-// then thread 0 solves A xi = -g by Cholesky (binary64) and applies
-// T <- exp(xi^) T; a matrix that is not positive definite leaves T as it is.
-// The step's sums, its starting pose and its xi are recorded at record.
-constexpr int SOLVE_THREADS = 256;
-__global__ void __launch_bounds__(SOLVE_THREADS) k_icp_solve(const double* __restrict__ partials, int blocks,
-                                                              double* __restrict__ pose, double* __restrict__ record) {
-    __shared__ double s[NSUM];
-    // warp w sums partials w, w + 8, ...: lane l the blocks l, l + 32, ... in
-    // order, then the lanes in a fixed shuffle pattern (deterministic)
-    const int lane = threadIdx.x & 31;
-    for (int k = threadIdx.x >> 5; k < NSUM; k += SOLVE_THREADS / 32) {
-        double v = 0.0;
-        for (int b = lane; b < blocks; b += 32) v += partials[(size_t)b * NSUM + k];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) s[k] = v;
-    }
+    if (!last) return;
+    __threadfence();
+    // lane l of warp w: sum l of blocks w, w + 8, ... in order, then the warps'
+    double v = 0.0;
+#pragma unroll 4
+    for (int b = warp; b < (int)gridDim.x; b += NW) v += __ldcg(partials + (size_t)b * NSLOT + lane);
+    red[warp][lane] = v;
     __syncthreads();
-    if (threadIdx.x != 0) return;
-    double A[36], g[6];
-    int k = 0;
+    if (warp != 0) return;
+    v = 0.0;
 #pragma unroll
-    for (int a = 0; a < 6; ++a)
-#pragma unroll
-        for (int b = a; b < 6; ++b, ++k) A[a * 6 + b] = A[b * 6 + a] = s[k];
-#pragma unroll
-    for (int a = 0; a < 6; ++a) g[a] = s[21 + a];
-    // record: sums (29), pose before the step (16), xi (6), solved flag (1)
-#pragma unroll
-    for (int i = 0; i < NSUM; ++i) record[i] = s[i];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) record[NSUM + i] = pose[i];
-    // fully unrolled (the arrays then live in registers, not in local
-    // memory); a pivot that is not positive marks the step unsolved and is
-    // replaced by 1 so the remaining arithmetic stays finite (its result is
-    // not used)
-    double Lc[36] = {0.0};
-    bool ok = true;
-#pragma unroll
-    for (int i = 0; i < 6; ++i)
-#pragma unroll
-        for (int j = 0; j <= i; ++j) {
-            double v = A[i * 6 + j];
-#pragma unroll
-            for (int q = 0; q < j; ++q) v -= Lc[i * 6 + q] * Lc[j * 6 + q];
-            if (i == j) {
-                if (!(v > 0.0)) {
-                    ok = false;
-                    v = 1.0;
-                }
-                Lc[i * 6 + i] = sqrt(v);
-            } else {
-                Lc[i * 6 + j] = v / Lc[j * 6 + j];
-            }
-        }
-    double xi[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    if (ok) {
-        double y[6];
-#pragma unroll
-        for (int i = 0; i < 6; ++i) {
-            double v = -g[i];
-#pragma unroll
-            for (int q = 0; q < i; ++q) v -= Lc[i * 6 + q] * y[q];
-            y[i] = v / Lc[i * 6 + i];
-        }
-#pragma unroll
-        for (int i = 5; i >= 0; --i) {
-            double v = y[i];
-#pragma unroll
-            for (int q = i + 1; q < 6; ++q) v -= Lc[q * 6 + i] * xi[q];
-            xi[i] = v / Lc[i * 6 + i];
-        }
-        // exp(xi^): Rodrigues rotation, V(phi) rho translation
-        const double* rho = xi;
-        const double* phi = xi + 3;
-        const double a2 = phi[0] * phi[0] + phi[1] * phi[1] + phi[2] * phi[2], a = sqrt(a2);
-        double cA, cB, cC;
-        if (a < 1e-4) {
-            cA = 1.0 - a2 / 6.0;
-            cB = 0.5 - a2 / 24.0;
-            cC = 1.0 / 6.0 - a2 / 120.0;
-        } else {
-            cA = sin(a) / a;
-            cB = (1.0 - cos(a)) / a2;
-            cC = (a - sin(a)) / (a2 * a);
-        }
-        const double W[9] = {0, -phi[2], phi[1], phi[2], 0, -phi[0], -phi[1], phi[0], 0};
-        double W2[9], Rm[9], Vm[9], tv[3], out[12];
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) {
-                double v = 0.0;
-#pragma unroll
-                for (int q = 0; q < 3; ++q) v += W[i * 3 + q] * W[q * 3 + j];
-                W2[i * 3 + j] = v;
-            }
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            const double I = (i % 4 == 0) ? 1.0 : 0.0;
-            Rm[i] = I + cA * W[i] + cB * W2[i];
-            Vm[i] = I + cB * W[i] + cC * W2[i];
-        }
-#pragma unroll
-        for (int i = 0; i < 3; ++i) tv[i] = Vm[i * 3] * rho[0] + Vm[i * 3 + 1] * rho[1] + Vm[i * 3 + 2] * rho[2];
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                double v = 0.0;
-#pragma unroll
-                for (int q = 0; q < 3; ++q) v += Rm[i * 3 + q] * pose[q * 4 + j];
-                out[i * 4 + j] = v + (j == 3 ? tv[i] : 0.0);
-            }
-#pragma unroll
-        for (int i = 0; i < 12; ++i) pose[i] = out[i];
-    }
-#pragma unroll
-    for (int i = 0; i < 6; ++i) record[NSUM + 16 + i] = xi[i];
-    record[NSUM + 22] = ok ? 1.0 : 0.0;
+    for (int w = 0; w < NW; ++w) v += red[w][lane];
+    S.s[lane] = v;
+    if (lane == 0) *finished = 0u;
+    __syncwarp();
+    icp_solve(S, pose, record, lane);
 }
 
 }  // namespace
@@ -313,26 +368,30 @@ cudaError_t launch_track_maps(const float* d, int w, int h, const float Kinv4[4]
     return cudaGetLastError();
 }
 
-// Blocks of a terms launch: one thread per pixel up to TRACK_MAX_BLOCKS
-// blocks, then each thread takes several pixels.  Each block reduces its 29
-// binary64 sums across its threads; with more blocks that reduction, not the
-// pixels, became the kernel's main cost (measured per tracked frame: 1024
-// blocks 4.34 ms, 608 and 320 4.35-4.38 ms, 152 3.88 ms, 114 3.96 ms, 76
-// 4.05 ms).
-constexpr int TRACK_MAX_BLOCKS = 152;  // one per SM of a GB300
+// Blocks of a step's launch: one thread per pixel up to one block per SM of a
+// GB300, then each thread takes several pixels.  Every block reduces its
+// threads' sums, so more blocks cost more than their pixels gain.
+constexpr int TRACK_MAX_BLOCKS = 152;
 int track_blocks(int npx) {
     const int want = (npx + TRACK_THREADS - 1) / TRACK_THREADS;
     return want < TRACK_MAX_BLOCKS ? (want > 0 ? want : 1) : TRACK_MAX_BLOCKS;
 }
 
+size_t track_partial_doubles(int npx) { return (size_t)track_blocks(npx) * NSLOT; }
 size_t track_record_doubles() { return NSUM + 16 + 6 + 1; }
 
-cudaError_t launch_track_step(const TrackLevel& L, double* pose, double* partials, double* record,
+cudaError_t launch_track_step(const TrackLevel& L, double* pose, double* partials, unsigned* finished, double* record,
                               cudaStream_t stream) {
-    const int blocks = track_blocks(L.w * L.h);
-    k_icp_terms<<<blocks, TRACK_THREADS, 0, stream>>>(L, pose, partials);
-    k_icp_solve<<<1, SOLVE_THREADS, 0, stream>>>(partials, blocks, pose, record);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)track_blocks(L.w * L.h));
+    cfg.blockDim = dim3(TRACK_THREADS);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_icp_step, L, pose, partials, finished, record);
 }
 
 }  // namespace tsdf

@@ -11,20 +11,28 @@ using namespace tsdf_host;
 
 namespace {
 
-// Temporary device buffers of one call, freed when it returns.
+// Temporary device buffers of one call, carved from one allocation (an
+// allocator call costs several microseconds of the host, and nothing is
+// queued before the buffers are there), freed when it returns.
 struct Scratchpad {
     tsdf_volume* v;
-    std::vector<void*> ptrs;
+    char* base = nullptr;
+    size_t used = 0;
     explicit Scratchpad(tsdf_volume* vol) : v(vol) {}
+    static size_t padded(size_t bytes) { return (bytes + 16 + 255) & ~(size_t)255; }
+    bool reserve(size_t bytes) {
+        base = static_cast<char*>(dev_alloc(v, bytes));
+        return base != nullptr;
+    }
     template <typename T>
     T* get(size_t n) {
-        void* p = dev_alloc(v, n * sizeof(T) + 16);
-        if (p) ptrs.push_back(p);
-        return static_cast<T*>(p);
+        T* p = reinterpret_cast<T*>(base + used);
+        used += padded(n * sizeof(T));
+        return p;
     }
     ~Scratchpad() {
         cudaStreamSynchronize(v->stream);
-        for (void* p : ptrs) dev_free(v, p);
+        if (base) dev_free(v, base);
     }
 };
 
@@ -79,10 +87,20 @@ extern "C" tsdf_status tsdf_track(tsdf_volume* v, const uint16_t* depth_mm, tsdf
     Scratchpad sp(v);
     const int W = dsz.width, H = dsz.height;
     cudaError_t e = cudaSuccess;
+    const bool staged = !is_device_ptr(depth_mm);
+    const size_t rec_n = tsdf::track_record_doubles();
+    size_t bytes = staged ? Scratchpad::padded((size_t)W * H * sizeof(uint16_t)) : 0;
+    for (int l = 0; l < p.levels; ++l) {
+        const size_t n = (size_t)(W >> l) * (H >> l) * sizeof(float);
+        bytes += Scratchpad::padded(n) + 4 * Scratchpad::padded(3 * n);
+    }
+    bytes += Scratchpad::padded(16 * sizeof(double)) + Scratchpad::padded(sizeof(unsigned)) +
+             Scratchpad::padded(tsdf::track_partial_doubles(W * H) * sizeof(double)) +
+             Scratchpad::padded((size_t)TSDF_TRACK_MAX_STEPS * rec_n * sizeof(double));
+    if (!sp.reserve(bytes)) return fail(v, TSDF_ERR_OOM, "track: buffers");
     const uint16_t* d_depth = depth_mm;
-    if (!is_device_ptr(depth_mm)) {
+    if (staged) {
         uint16_t* buf = sp.get<uint16_t>((size_t)W * H);
-        if (!buf) return fail(v, TSDF_ERR_OOM, "track: depth staging");
         e = cudaMemcpyAsync(buf, depth_mm, (size_t)W * H * sizeof(uint16_t), cudaMemcpyHostToDevice, v->stream);
         d_depth = buf;
     }
@@ -96,14 +114,13 @@ extern "C" tsdf_status tsdf_track(tsdf_volume* v, const uint16_t* depth_mm, tsdf
         Nl[l] = sp.get<float>(3 * n);
         PVl[l] = sp.get<float>(3 * n);
         PNl[l] = sp.get<float>(3 * n);
-        if (!dl[l] || !Vl[l] || !Nl[l] || !PVl[l] || !PNl[l]) return fail(v, TSDF_ERR_OOM, "track: level buffers");
     }
-    const size_t rec_n = tsdf::track_record_doubles();
     double* pose = sp.get<double>(16);
-    double* partials = sp.get<double>((size_t)tsdf::track_blocks(W * H) * 29);
+    unsigned* finished = sp.get<unsigned>(1);
+    double* partials = sp.get<double>(tsdf::track_partial_doubles(W * H));
     double* records = sp.get<double>((size_t)TSDF_TRACK_MAX_STEPS * rec_n);
-    if (!pose || !partials || !records) return fail(v, TSDF_ERR_OOM, "track: step buffers");
     if (e == cudaSuccess) e = cudaMemcpyAsync(pose, T_init, 16 * sizeof(double), cudaMemcpyHostToDevice, v->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(finished, 0, sizeof *finished, v->stream);
     if (e == cudaSuccess) e = tsdf::launch_track_pyramid(d_depth, W, H, p.levels, dl, v->stream);
     if (e == cudaSuccess) e = tsdf::launch_ray_map(v->vol.summ, v->nb, v->plain_f, v->scr.ray_map, v->stream);
     if (e != cudaSuccess) return cuda_fail(v, e, "track: pyramid");
@@ -152,7 +169,7 @@ extern "C" tsdf_status tsdf_track(tsdf_volume* v, const uint16_t* depth_mm, tsdf
         L.PN = PNl[l];
         for (int it = 0; it < p.iterations[l]; ++it, ++step) {
             step_level[step] = l;
-            e = tsdf::launch_track_step(L, pose, partials, records + (size_t)step * rec_n, v->stream);
+            e = tsdf::launch_track_step(L, pose, partials, finished, records + (size_t)step * rec_n, v->stream);
             if (e != cudaSuccess) return cuda_fail(v, e, "track: step");
         }
     }
