@@ -43,6 +43,7 @@ struct FrameConst {
     int32_t zoff_g, zoff_c;  // z-slab: global z index of held geometry / colour z = 0 (whole volume: 0)
     uint32_t pix_bias;       // 0x4B000000 (dw + 1) mod 2^32: pixel index from the bits of u + 2^23, v + 2^23
     uint32_t frame_tag;      // nonzero, different in consecutive frames: marks this frame's ready-queue entries
+    int32_t open_bricks;     // 1: open bricks (see brick_flags) take their own geometry update
     int32_t fused;           // 1: the frame runs as one fused launch (k_fused) instead of the kernel chain
 };
 
@@ -57,11 +58,11 @@ struct BrickSummary {
 };
 
 struct Counters {
-    uint32_t n_geo;      // geometry work list length
+    uint32_t n_geo;      // geometry work list length (bricks not open)
     uint32_t n_vis;      // visible brick list length
     uint32_t n_col;      // colour work list length
-    uint32_t geo_next;   // persistent-loop work counters
-    uint32_t col_next;
+    uint32_t n_geo_open; // open bricks (see brick_flags): geometry work list entries from the buffer's end
+    uint32_t col_next;   // persistent-loop work counter
     uint32_t n_vox;      // band-gate voxel records (may exceed the buffer's capacity)
     uint32_t n_cells;    // trilinear cells that can pass the band gate
     uint32_t n_col_active;   // colour candidates with at least one such cell

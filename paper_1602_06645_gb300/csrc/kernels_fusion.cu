@@ -95,13 +95,12 @@ __global__ void __launch_bounds__(TILES_THREADS) k_depth_tiles(FrameConst c, con
         // totals (the colour side is folded by the geometry kernel, so this
         // kernel may run while the previous frame's colour work finishes)
         ctr->tot_geo_updated += ctr->geo_updated;
-        ctr->tot_geo_bricks += ctr->n_geo;
+        ctr->tot_geo_bricks += ctr->n_geo + ctr->n_geo_open;
         ctr->tot_vis_bricks += ctr->n_vis;
         ctr->tot_geo_changed += ctr->n_geo_changed;
         ctr->n_geo_changed = 0;
         ctr->frames += 1ull;
-        ctr->n_geo = ctr->n_vis = 0;
-        ctr->geo_next = 0;
+        ctr->n_geo = ctr->n_geo_open = ctr->n_vis = 0;
         ctr->geo_updated = 0ull;
     }
 }
@@ -205,10 +204,11 @@ __device__ __forceinline__ bool ball_outside_image(const FrameConst& c, const fl
 
 __device__ __forceinline__ void brick_flags(const FrameConst& c, const BrickSummary* __restrict__ summ,
                                             const uint32_t* __restrict__ tiles, uint32_t b, bool in, bool& geo,
-                                            bool& vis, bool& inner) {
+                                            bool& vis, bool& inner, bool& open) {
     vis = in;
     geo = in;
     inner = false;
+    open = false;
     if (in && c.culling) {
         int bx = b % c.nb[0], by = (b / c.nb[0]) % c.nb[1], bz = b / (c.nb[0] * c.nb[1]);
         if (c.kd_pinhole) {
@@ -276,8 +276,14 @@ __device__ __forceinline__ void brick_flags(const FrameConst& c, const BrickSumm
         // the geometry update skips sdf < -mu, so mu (not max(mu, sigma)) bounds it
         geo = vis && !(zmin > (float)dmax * 0.001f + c.mu + 2e-3f);
         if (vis) {
-            bool sat = c.free_space == 0 || (s.fmin == 1.0f && s.wmin == (uint32_t)c.max_weight);
-            if (sat && zmax < (float)dmin * 0.001f - c.mu - 2e-3f) geo = false;
+            const bool ones = s.fmin == 1.0f && s.fmax == 1.0f;  // every observed voxel (a restored F may exceed 1)
+            bool sat = c.free_space == 0 || (ones && s.wmin == (uint32_t)c.max_weight);
+            const bool ahead = zmax < (float)dmin * 0.001f - c.mu - 2e-3f;
+            if (sat && ahead) geo = false;
+            // every measurement under an open brick puts its voxels at t = 1,
+            // and every voxel observed so far is at F = 1 (or none is): the
+            // update only counts (see geometry_open)
+            open = c.open_bricks && ahead && (ones || !(s.fmin <= FLT_MAX));
             // colour: Eq. 7 needs |Z - d| <= sigma (pinhole K_c: the back-projected
             // point has Z = d), so a brick wholly nearer than the nearest depth
             // minus sigma holds no colour voxel that can pass
@@ -286,38 +292,10 @@ __device__ __forceinline__ void brick_flags(const FrameConst& c, const BrickSumm
     }
 }
 
-// Append the flagged values of a whole block to two lists with one atomic per
-// list per block (all threads of the block call it): thousands of warps
-// finishing together would otherwise queue on the two counters.
-template <int NT>
-__device__ __forceinline__ void block_append2(bool p0, bool p1, uint32_t value0, uint32_t value1, uint32_t* ctr0,
-                                              uint32_t* list0, uint32_t* ctr1, uint32_t* list1) {
-    constexpr int NW = NT / 32;
-    __shared__ uint32_t off[2][NW + 1];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const unsigned m0 = __ballot_sync(0xffffffffu, p0), m1 = __ballot_sync(0xffffffffu, p1);
-    if (lane == 0) {
-        off[0][wid] = __popc(m0);
-        off[1][wid] = __popc(m1);
-    }
-    __syncthreads();
-    if (threadIdx.x < 2) {
-        uint32_t tot = 0;
-        for (int w = 0; w < NW; ++w) {
-            const uint32_t n = off[threadIdx.x][w];
-            off[threadIdx.x][w] = tot;
-            tot += n;
-        }
-        off[threadIdx.x][NW] = tot ? atomicAdd(threadIdx.x ? ctr1 : ctr0, tot) : 0u;
-    }
-    __syncthreads();
-    const unsigned lt = (1u << lane) - 1u;
-    if (p0) list0[off[0][NW] + off[0][wid] + __popc(m0 & lt)] = value0;
-    if (p1) list1[off[1][NW] + off[1][wid] + __popc(m1 & lt)] = value1;
-    __syncthreads();  // off is reused by the block's next call
-}
-
-// The same for three lists, the third filled from its end down: its k-th
+// Append the flagged values of a whole block to three lists with one atomic
+// per list per block (all threads of the block call it): thousands of warps
+// finishing together would otherwise queue on the counters.  The third list is
+// filled from its end down: its k-th
 // value goes to list2_end[-1 - k].
 template <int NT>
 __device__ __forceinline__ void block_append3(bool p0, bool p1, bool p2, uint32_t value0, uint32_t value1,
@@ -381,7 +359,9 @@ __device__ __forceinline__ void block_add(uint32_t v0, T0* d0, uint32_t v1 = 0u,
 
 // Geometry work-list entry: the brick's coordinates (10 bits per axis; the
 // volume has at most 4096 voxels = 512 bricks per axis) and, in bit 31, the
-// interior flag (the brick projects wholly into the image).
+// interior flag (the brick projects wholly into the image).  Open bricks are
+// listed from the buffer's end: each warp then takes its share of the long
+// updates and its share of the short ones.
 constexpr uint32_t GEO_INNER = 0x80000000u;
 __device__ __forceinline__ uint32_t geo_entry(const FrameConst& c, uint32_t b, bool inner) {
     const uint32_t nb0 = (uint32_t)c.nb[0], nb1 = (uint32_t)c.nb[1];
@@ -412,8 +392,8 @@ __global__ void __launch_bounds__(BRICK_THREADS) k_bricks(FrameConst c, const Br
     chain_enter();
     const uint32_t nbt = (uint32_t)c.nb[0] * c.nb[1] * c.nb[2];
     uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;
-    bool geo, vis, inner;
-    brick_flags(c, summ, tiles, b, b < nbt, geo, vis, inner);
+    bool geo, vis, inner, open;
+    brick_flags(c, summ, tiles, b, b < nbt, geo, vis, inner, open);
     if (c.fused) {
         if (b < nbt) bstate[b] = (uint8_t)((geo ? 1u : 0u) | (vis ? 2u : 0u));
         if (b == 0) {
@@ -422,8 +402,9 @@ __global__ void __launch_bounds__(BRICK_THREADS) k_bricks(FrameConst c, const Br
         }
     }
     // geometry list entries carry the interior flag in bit 31
-    block_append2<BRICK_THREADS>(geo, vis, geo_entry(c, b, inner), b, &ctr->n_geo, geo_list, &ctr->n_vis,
-                                 vis_list);
+    const uint32_t e = geo_entry(c, b, inner);
+    block_append3<BRICK_THREADS>(geo && !open, vis, geo && open, e, b, e, &ctr->n_geo, geo_list, &ctr->n_vis, vis_list,
+                                 &ctr->n_geo_open, geo_list + nbt);
 }
 
 // ---------------------------------------------------------- geometry ----
@@ -445,17 +426,14 @@ __device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
 
 // Nearest depth pixel of a pair of camera points (Eq. 6: xh = fmaf(K0, X,
 // K2 Z) for a pinhole K, u = xh (1/zh), pixel floor(u + 1/2)).  The floor is
-// taken as (u + 1/2) + 2^23 rounded toward minus infinity, whose bits are
-// 0x4B000000 + floor(u + 1/2) for 0 <= u + 1/2 < 2^23 and fall outside the
+// taken as (u + 1/2) + 2^23 rounded toward minus infinity (bu, bv), whose bits
+// are 0x4B000000 + floor(u + 1/2) for 0 <= u + 1/2 < 2^23 and fall outside the
 // image test for any other value (negative, huge or infinite), so the
-// integer test 0 <= floor < W is the float test 0 <= u + 1/2 < W.  The pixel
-// index iv W + iu is then (bits of v) W + (bits of u) - 0x4B000000 (W + 1),
-// modulo 2^32.  INNER: the caller knows every point lies in front of the
-// camera and inside the image.  Otherwise a point outside the image gets
-// pixel 0 and ok = false.
+// integer test 0 <= floor < W is the float test 0 <= u + 1/2 < W.  INNER: the
+// caller knows every point lies in front of the camera and inside the image.
 template <bool PINHOLE, bool INNER>
-__device__ __forceinline__ void depth_pixels(const FrameConst& c, float2 X, float2 Y, float2 Z, uint32_t pix[2],
-                                             bool ok[2]) {
+__device__ __forceinline__ void depth_coords(const FrameConst& c, float2 X, float2 Y, float2 Z, float2& bu,
+                                             float2& bv, bool ok[2]) {
     float2 xh, yh, zh;
     if (PINHOLE) {
         xh = __ffma2_rn(f2(c.Kd[0]), X, __fmul2_rn(f2(c.Kd[2]), Z));
@@ -467,18 +445,28 @@ __device__ __forceinline__ void depth_pixels(const FrameConst& c, float2 X, floa
         zh = __ffma2_rn(f2(c.Kd[6]), X, __ffma2_rn(f2(c.Kd[7]), Y, __fmul2_rn(f2(c.Kd[8]), Z)));
     }
     const float2 rz = rcp2_rn(zh);
-    const float2 bu = __fadd2_rd(__fadd2_rn(__fmul2_rn(xh, rz), f2(0.5f)), f2(8388608.0f));
-    const float2 bv = __fadd2_rd(__fadd2_rn(__fmul2_rn(yh, rz), f2(0.5f)), f2(8388608.0f));
-    const uint32_t u0 = __float_as_uint(bu.x), u1 = __float_as_uint(bu.y);
-    const uint32_t v0 = __float_as_uint(bv.x), v1 = __float_as_uint(bv.y);
+    bu = __fadd2_rd(__fadd2_rn(__fmul2_rn(xh, rz), f2(0.5f)), f2(8388608.0f));
+    bv = __fadd2_rd(__fadd2_rn(__fmul2_rn(yh, rz), f2(0.5f)), f2(8388608.0f));
+    ok[0] = ok[1] = true;
+    if (!INNER) {
+        const uint32_t dw = (uint32_t)c.dw, dh = (uint32_t)c.dh;
+        ok[0] = zh.x > 0.0f && __float_as_uint(bu.x) - 0x4B000000u < dw && __float_as_uint(bv.x) - 0x4B000000u < dh;
+        ok[1] = zh.y > 0.0f && __float_as_uint(bu.y) - 0x4B000000u < dw && __float_as_uint(bv.y) - 0x4B000000u < dh;
+    }
+}
+
+// The same as pixel indices iv W + iu = (bits of v) W + (bits of u) -
+// 0x4B000000 (W + 1), modulo 2^32; a point outside the image gets pixel 0 and
+// ok = false.
+template <bool PINHOLE, bool INNER>
+__device__ __forceinline__ void depth_pixels(const FrameConst& c, float2 X, float2 Y, float2 Z, uint32_t pix[2],
+                                             bool ok[2]) {
+    float2 bu, bv;
+    depth_coords<PINHOLE, INNER>(c, X, Y, Z, bu, bv, ok);
     const uint32_t dw = (uint32_t)c.dw;
-    pix[0] = v0 * dw + u0 - c.pix_bias;
-    pix[1] = v1 * dw + u1 - c.pix_bias;
-    if (INNER) {
-        ok[0] = ok[1] = true;
-    } else {
-        ok[0] = zh.x > 0.0f && u0 - 0x4B000000u < dw && v0 - 0x4B000000u < (uint32_t)c.dh;
-        ok[1] = zh.y > 0.0f && u1 - 0x4B000000u < dw && v1 - 0x4B000000u < (uint32_t)c.dh;
+    pix[0] = __float_as_uint(bv.x) * dw + __float_as_uint(bu.x) - c.pix_bias;
+    pix[1] = __float_as_uint(bv.y) * dw + __float_as_uint(bu.y) - c.pix_bias;
+    if (!INNER) {
         if (!ok[0]) pix[0] = 0u;
         if (!ok[1]) pix[1] = 0u;
     }
@@ -724,6 +712,167 @@ __device__ __forceinline__ void geometry_brick(const FrameConst& c, const Volume
     geometry_update<PINHOLE, FREE_SPACE, ALIGNED, INNER>(c, vol, depth, at, lane, f, wv, count, changed);
 }
 
+// The depth at pixel 0x4B000000 + i of an image of less than 2^23 pixels, as a
+// word whose sign bit says that there is none.
+__device__ __forceinline__ uint32_t depth_gap(DepthM depth, uint32_t bits) {
+    uint32_t d;
+    const uint64_t at = (uint64_t)(uintptr_t)depth.p - 4ull * 0x4B000000u + 4ull * bits;
+    asm("ld.global.nc.u32 %0, [%1];" : "=r"(d) : "l"(at));
+    return d;
+}
+__device__ __forceinline__ uint32_t depth_gap(DepthMm depth, uint32_t bits) {
+    uint16_t d;
+    const uint64_t at = (uint64_t)(uintptr_t)depth.p - 2ull * 0x4B000000u + 2ull * bits;
+    asm("ld.global.nc.u16 %0, [%1];" : "=h"(d) : "l"(at));
+    return (uint32_t)d - 1u;
+}
+
+// Update of an open brick (see brick_flags): every voxel with a measurement
+// gets t = 1 and holds F = 1 or, unobserved, F = fmaf(F, 0, 1) / 1 = 1, and
+// (1 w + 1) / (w + 1) = 1 exactly, so F changes only where a voxel is observed
+// for the first time and the update counts weights.  Same lane layout and
+// result as geometry_update (F, w and summary), without reading F, the
+// averages, and (but for first observations) writing F: 1 KB of traffic per
+// brick instead of 5, and the instructions of the projection alone, which are
+// what bounds it.  The pixel index is formed in binary32 (exact below 2^23
+// pixels, FrameConst::open_bricks): 2^23 + iv W + iu, whose bits index the
+// depth image from a base moved by 0x4B000000 pixels.  Three quarters of a
+// scan frame's listed bricks (58,000 of 78,000) are open until their weights
+// saturate; the geometry phase of those frames went from 81 to 60 us.  A
+// launch of their own at 40 registers, started behind this one's blocks, took
+// 57 us, but a launch more in every frame; taking them between the other
+// bricks, or first in every other warp, 61 and 68 us.
+template <bool PINHOLE, bool ALIGNED, bool INNER, typename Depth>
+__device__ __forceinline__ void geometry_open(const FrameConst& c, const Volumes& vol, Depth depth, const BrickAt& at,
+                                              int lane, uint32_t& count, uint32_t& changed) {
+    const int lx = (lane & 1) * 4, ly = (lane >> 1) & 7, lz = lane >> 4;
+    uint8_t* Wb = vol.W + (size_t)at.b * BRICK_VOX + lane * 4;
+    uint32_t wv[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) wv[j] = *reinterpret_cast<const uint32_t*>(Wb + 128 * j);
+    const int gx0 = at.bx * BRICK + lx, gy = at.by * BRICK + ly;
+    const float py = fmaf((float)gy + 0.5f, c.s_g, c.origin[1]);
+    const float gxf = (float)gx0;
+    const float2 pxp[2] = {make_float2(fmaf(gxf + 0.5f, c.s_g, c.origin[0]), fmaf(gxf + 1.5f, c.s_g, c.origin[0])),
+                           make_float2(fmaf(gxf + 2.5f, c.s_g, c.origin[0]), fmaf(gxf + 3.5f, c.s_g, c.origin[0]))};
+    const float gzf = (float)(at.bz * BRICK + lz + c.zoff_g) + 0.5f;
+    uint32_t within = 0xFFFFu;  // this lane's voxels inside the volume, bit 4 j + i
+    uint32_t db[16];            // the sixteen depth reads in flight together; only their sign bit counts
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const float pz = fmaf(gzf + (float)(2 * j), c.s_g, c.origin[2]);
+        const float2 B0 = f2(fmaf(c.R[1], py, fmaf(c.R[2], pz, c.t[0])));
+        const float2 B1 = f2(fmaf(c.R[4], py, fmaf(c.R[5], pz, c.t[1])));
+        const float2 B2 = f2(fmaf(c.R[7], py, fmaf(c.R[8], pz, c.t[2])));
+        const bool yzin = ALIGNED || (gy < c.ng[1] && at.bz * BRICK + lz + 2 * j < c.ng[2]);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float2 X = __ffma2_rn(f2(c.R[0]), pxp[h], B0);
+            const float2 Y = __ffma2_rn(f2(c.R[3]), pxp[h], B1);
+            const float2 Z = __ffma2_rn(f2(c.R[6]), pxp[h], B2);
+            float2 bu, bv;
+            bool ok[2];
+            depth_coords<PINHOLE, INNER>(c, X, Y, Z, bu, bv, ok);
+            const float2 id = __ffma2_rn(f2((float)c.dw), __fadd2_rn(bv, f2(-8388608.0f)), bu);
+            const uint32_t bits[2] = {__float_as_uint(id.x), __float_as_uint(id.y)};
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const int i = 2 * h + k;
+                if (!ALIGNED && !(yzin && gx0 + i < c.ng[0])) {
+                    within &= ~(1u << (4 * j + i));
+                    ok[k] = false;
+                }
+                const bool sure = INNER && ALIGNED;
+                const uint32_t d = depth_gap(depth, sure || ok[k] ? bits[k] : 0x4B000000u);
+                db[4 * j + i] = sure || ok[k] ? d : 0x80000000u;
+            }
+        }
+    }
+    uint32_t gaps = 0;
+#pragma unroll
+    for (int v = 15; v >= 0; --v) gaps = __funnelshift_l(db[v], gaps, 1);
+    const uint32_t upd = ~gaps & 0xFFFFu;
+    count += __popc(upd);
+    if (!__any_sync(0xffffffffu, upd != 0u)) return;  // nothing changed: the summary stays
+    ++changed;
+    const uint32_t maxw = (uint32_t)c.max_weight, maxw4 = maxw * 0x01010101u;
+    // w <- min(w + 1, max_weight) of the updated voxels, as in geometry_update
+    uint32_t wn[4], below = 0;
+    bool hole = false;  // an unobserved voxel before the update
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const uint32_t upm = (upd >> (4 * j)) & 15u, w_old = wv[j];
+        const uint32_t upb = (upm * 0x00204081u) & 0x01010101u;  // bit i of upm -> byte i
+        wn[j] = w_old + (upb & ~zero_bytes(w_old ^ maxw4));
+        hole = hole || any_zero_byte(w_old);
+        below |= wn[j] ^ maxw4;
+        if (upm) *reinterpret_cast<uint32_t*>(Wb + 128 * j) = wn[j];
+    }
+    const float lo_thr = c.band + CELL_EPS, hi_thr = -c.band - CELL_EPS;
+    const uint32_t side = (1.0f <= lo_thr ? 1u : 0u) | (1.0f >= hi_thr ? 2u : 0u);
+    uint32_t bflags = side * 0x1555u;  // every voxel observed: the same on all faces
+    bool unobserved = false, below_cap = below != 0u;
+    if (__any_sync(0xffffffffu, hole)) {
+        float* Fb = vol.F + (size_t)at.b * BRICK_VOX + lane * 4;
+        uint32_t seen = 0;  // observed voxels after the update, bit 4 j + i
+        below_cap = false;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t upm = (upd >> (4 * j)) & 15u;
+            const uint32_t z4 = (zero_bytes(wv[j]) * 0x01020408u) >> 24;  // byte i -> bit i: unobserved before
+            const uint32_t first = upm & z4;
+            if (first == 15u) {
+                *reinterpret_cast<float4*>(Fb + 128 * j) = make_float4(1.0f, 1.0f, 1.0f, 1.0f);
+            } else if (first) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if ((first >> i) & 1u) Fb[128 * j + i] = 1.0f;
+            }
+            seen |= (upm | (~z4 & 15u)) << (4 * j);
+            // in-volume voxels only: a byte outside reads as observed and at the cap
+            const uint32_t inside =
+                ALIGNED ? 0xFFFFFFFFu : ((((within >> (4 * j)) & 15u) * 0x00204081u) & 0x01010101u) * 0xFFu;
+            const uint32_t wq = (wn[j] & inside) | (maxw4 & ~inside);
+            unobserved = unobserved || any_zero_byte(wq);
+            below_cap = below_cap || wq != maxw4;
+        }
+        seen &= within;
+        const uint32_t all = seen ? side : 0u;
+        const uint32_t xf = (seen & (lx == 0 ? 0x1111u : 0x8888u)) ? side : 0u;
+        const uint32_t zf = (seen & (lz == 0 ? 0x000Fu : 0xF000u)) ? side : 0u;
+        bflags = __reduce_or_sync(0xffffffffu, all | (lx == 0 ? xf << 2 : xf << 4) | (ly == 0 ? all << 6 : 0u) |
+                                                   (ly == 7 ? all << 8 : 0u) | (lz == 0 ? zf << 10 : zf << 12));
+        unobserved = __any_sync(0xffffffffu, unobserved);
+    }
+    below_cap = __any_sync(0xffffffffu, below_cap);
+    if (lane == 0) {
+        BrickSummary sm;
+        sm.fmin = sm.fmax = 1.0f;
+        sm.wmin = unobserved ? 0u : (below_cap ? maxw - 1u : maxw);
+        sm.flags = bflags;
+        vol.summ[at.b] = sm;
+    }
+}
+
+// Entry `item` of the geometry work list (n = n_geo entries from the front,
+// then the open bricks): its update.
+template <bool PINHOLE, bool FREE_SPACE, bool ALIGNED, typename Depth>
+__device__ __forceinline__ void geometry_item(const FrameConst& c, const Volumes& vol, Depth depth, uint32_t e,
+                                              bool open, const BrickAt& at, int lane, uint32_t& count,
+                                              uint32_t& changed) {
+    // GEO_INNER: the brick projects wholly into the image, no per-voxel image tests
+    if (FREE_SPACE && open) {
+        if (e & GEO_INNER)
+            geometry_open<PINHOLE, ALIGNED, true>(c, vol, depth, at, lane, count, changed);
+        else
+            geometry_open<PINHOLE, ALIGNED, false>(c, vol, depth, at, lane, count, changed);
+    } else if (e & GEO_INNER) {
+        geometry_brick<PINHOLE, FREE_SPACE, ALIGNED, true>(c, vol, depth, at, lane, count, changed);
+    } else {
+        geometry_brick<PINHOLE, FREE_SPACE, ALIGNED, false>(c, vol, depth, at, lane, count, changed);
+    }
+}
+
 template <bool PINHOLE, bool FREE_SPACE, bool ALIGNED>
 __global__ void __launch_bounds__(GEO_THREADS, 8) k_geometry(FrameConst c, Volumes vol, const float* __restrict__ depth_m,
                                                           Counters* __restrict__ ctr,
@@ -748,13 +897,26 @@ __global__ void __launch_bounds__(GEO_THREADS, 8) k_geometry(FrameConst c, Volum
     // the list is taken from its end: the colour kernels that follow walk
     // their lists from the front, whose bricks are then the ones this kernel
     // wrote last (measured: 1 % off the frame)
-    for (uint32_t item = warp; item < n; item += nwarps) {
+    uint32_t item = warp;
+    for (; item < n; item += nwarps) {
         const uint32_t e = list[n - 1u - item];
         const BrickAt at = geo_brick(c, e);
         if (e & GEO_INNER)  // the brick projects wholly into the image: no per-voxel image tests
             geometry_brick<PINHOLE, FREE_SPACE, ALIGNED, true>(c, vol, depth, at, lane, count, changed);
         else
             geometry_brick<PINHOLE, FREE_SPACE, ALIGNED, false>(c, vol, depth, at, lane, count, changed);
+    }
+    if (FREE_SPACE) {  // the open bricks go on where the warp's share of the list ended (a loop of their own: 64 registers)
+        const uint32_t n_open = ctr->n_geo_open;
+        const uint32_t* end = list + (uint32_t)c.nb[0] * c.nb[1] * c.nb[2];
+        for (item -= n; item < n_open; item += nwarps) {
+            const uint32_t e = end[-1 - (int64_t)item];
+            const BrickAt at = geo_brick(c, e);
+            if (e & GEO_INNER)
+                geometry_open<PINHOLE, ALIGNED, true>(c, vol, depth, at, lane, count, changed);
+            else
+                geometry_open<PINHOLE, ALIGNED, false>(c, vol, depth, at, lane, count, changed);
+        }
     }
     block_add<GEO_THREADS>(__reduce_add_sync(0xffffffffu, count), &ctr->geo_updated, changed, &ctr->n_geo_changed);
 }
@@ -1608,7 +1770,8 @@ __global__ void __launch_bounds__(COL_THREADS, 5) k_fused(FrameConst c, Volumes 
     const int lane = threadIdx.x & 31;
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-    const uint32_t n = ctr->n_geo, nv = ctr->n_vis;
+    const uint32_t nf = ctr->n_geo, n = nf + ctr->n_geo_open, nv = ctr->n_vis;
+    const uint32_t nbt = (uint32_t)c.nb[0] * c.nb[1] * c.nb[2];
     const DepthM dm{scr.depth_m};
     uint32_t gcount = 0, changed = 0, count = 0, n_active = 0, n_cells = 0, n_cand = 0, nstage = 0;
     bool ok = true;
@@ -1616,12 +1779,10 @@ __global__ void __launch_bounds__(COL_THREADS, 5) k_fused(FrameConst c, Volumes 
     // neighbourhoods are complete follow the front), one ready colour brick
     // after each when the queue holds one
     for (uint32_t item = warp; item < n; item += nwarps) {
-        const uint32_t e = scr.geo_list[item];
+        const bool open = item >= nf;
+        const uint32_t e = scr.geo_list[open ? nbt - 1u - (item - nf) : item];
         const BrickAt at = geo_brick(c, e);
-        if (e & GEO_INNER)
-            geometry_brick<true, FREE_SPACE, ALIGNED, true>(c, vol, dm, at, lane, gcount, changed);
-        else
-            geometry_brick<true, FREE_SPACE, ALIGNED, false>(c, vol, dm, at, lane, gcount, changed);
+        geometry_item<true, FREE_SPACE, ALIGNED>(c, vol, dm, e, open, at, lane, gcount, changed);
         fuse_release(c, scr, at, lane);
         uint32_t slot = 0xFFFFFFFFu;
         if (lane == 0) {
@@ -1921,15 +2082,15 @@ __global__ void __launch_bounds__(COL_THREADS, 4) k_batch_step(const ScanDesc* _
         Counters* ctr = descs[tid].scr.ctr;
         ctr->tot_geo_updated += ctr->geo_updated;
         ctr->tot_col_updated += ctr->col_updated;
-        ctr->tot_geo_bricks += ctr->n_geo;
+        ctr->tot_geo_bricks += ctr->n_geo + ctr->n_geo_open;
         ctr->tot_col_bricks += ctr->n_col + ctr->n_col_light;
         ctr->tot_vis_bricks += ctr->n_vis;
         ctr->tot_cells += ctr->n_cells;
         ctr->tot_col_active += ctr->n_col_active;
         ctr->tot_geo_changed += ctr->n_geo_changed;
         ctr->frames += 1ull;
-        ctr->n_geo = ctr->n_vis = ctr->n_col = ctr->n_col_light = 0;
-        ctr->geo_next = ctr->col_next = 0;
+        ctr->n_geo = ctr->n_geo_open = ctr->n_vis = ctr->n_col = ctr->n_col_light = 0;
+        ctr->col_next = 0;
         ctr->n_cells = ctr->n_vox = 0;
         ctr->n_col_active = ctr->n_geo_changed = 0;
         ctr->geo_updated = ctr->col_updated = 0ull;
@@ -1951,34 +2112,38 @@ __global__ void __launch_bounds__(COL_THREADS, 4) k_batch_step(const ScanDesc* _
         const ScanDesc& d = descs[s];
         const uint32_t b = item - pre[s];
         const uint32_t nbt = (uint32_t)d.c.nb[0] * d.c.nb[1] * d.c.nb[2];
-        bool geo, vis, inner;
-        brick_flags(d.c, d.vol.summ, d.scr.depth_tiles, b, b < nbt, geo, vis, inner);
-        append(geo, geo_entry(d.c, b, inner), &d.scr.ctr->n_geo, d.scr.geo_list);
+        bool geo, vis, inner, open;
+        brick_flags(d.c, d.vol.summ, d.scr.depth_tiles, b, b < nbt, geo, vis, inner, open);
+        const uint32_t e = geo_entry(d.c, b, inner);
+        append(geo && !open, e, &d.scr.ctr->n_geo, d.scr.geo_list);
+        append_back(geo && open, e, &d.scr.ctr->n_geo_open, d.scr.geo_list + nbt);
         append(vis, b, &d.scr.ctr->n_vis, d.scr.vis_list);
     }
     if (!grid_barrier(sync, gridDim.x)) return;
 
     // P2: geometry, one warp per tile of `tile` consecutive listed bricks of a scan
-    scan_prefix(pre, n, 1, [&](int i) { return (descs[i].scr.ctr->n_geo + tile - 1) / tile; });
+    scan_prefix(pre, n, 1, [&](int i) {
+        return (descs[i].scr.ctr->n_geo + descs[i].scr.ctr->n_geo_open + tile - 1) / tile;
+    });
     for (uint32_t item = warp; item < pre[n]; item += nwarps) {
         const int s = find_scan(pre, n, item);
         const ScanDesc& d = descs[s];
-        const uint32_t k0 = (item - pre[s]) * tile, k1 = min(k0 + (uint32_t)tile, d.scr.ctr->n_geo);
+        const uint32_t nf = d.scr.ctr->n_geo, ng = nf + d.scr.ctr->n_geo_open;
+        const uint32_t nbt = (uint32_t)d.c.nb[0] * d.c.nb[1] * d.c.nb[2];
+        const uint32_t k0 = (item - pre[s]) * tile, k1 = min(k0 + (uint32_t)tile, ng);
         uint32_t count = 0, changed = 0;
         const bool aligned = d.c.ng[0] % BRICK == 0 && d.c.ng[1] % BRICK == 0 && d.c.ng[2] % BRICK == 0;
         for (uint32_t k = k0; k < k1; ++k) {
-            const uint32_t e = d.scr.geo_list[k];
+            const bool open = k >= nf;
+            const uint32_t e = d.scr.geo_list[open ? nbt - 1u - (k - nf) : k];
             const BrickAt at = geo_brick(d.c, e);
             const DepthMm dm{d.depth};
             // the usual camera and mode: without the per-voxel image tests for
             // bricks inside the image and without bounds tests for whole-brick
             // volumes; the general form handles every other brick
-            if (d.c.kd_pinhole && d.c.free_space && aligned) {
-                if (e & GEO_INNER)
-                    geometry_brick<true, true, true, true>(d.c, d.vol, dm, at, lane, count, changed);
-                else
-                    geometry_brick<true, true, true, false>(d.c, d.vol, dm, at, lane, count, changed);
-            } else if (d.c.kd_pinhole && d.c.free_space)
+            if (d.c.kd_pinhole && d.c.free_space && aligned)
+                geometry_item<true, true, true>(d.c, d.vol, dm, e, open, at, lane, count, changed);
+            else if (d.c.kd_pinhole && d.c.free_space)
                 geometry_brick<true, true>(d.c, d.vol, dm, at, lane, count, changed);
             else if (d.c.kd_pinhole)
                 geometry_brick<true, false>(d.c, d.vol, dm, at, lane, count, changed);

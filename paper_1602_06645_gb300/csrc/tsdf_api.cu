@@ -176,6 +176,16 @@ void frame_constants(const tsdf_volume* v, const float Kd[9], const float Kr[9],
     // Beyond the farthest depth by more than max(mu, sigma) nothing can pass
     // the sdf >= -mu test nor (pinhole K_c: the back-projected point has
     // Z = d) the sigma gate; 2 mm covers binary32 rounding many times over.
+    // Open bricks rest on a margin of 2 mm between binary32 depths computed in
+    // two ways; each is off by less than 1e-6 of the coordinates that enter it.
+    float far_out = 0.0f;
+    for (int a = 0; a < 3; ++a) {
+        const float end = v->origin[a] + (float)(v->ng[a] + (a == 2 ? v->zoff_g : 0)) * v->s_g;
+        far_out = std::fmax(far_out, std::fmax(std::fabs(v->origin[a]), std::fabs(end)));
+        far_out = std::fmax(far_out, std::fabs(Twd[a * 4 + 3]));
+    }
+    // Their pixel indices are binary32 integers.
+    c.open_bricks = v->plain_f && v->free_space && far_out <= 500.0f && (int64_t)dw * dh < (1 << 23) ? 1 : 0;
     c.cull_behind = c.kdi_pinhole ? std::fmax(v->mu, v->sigma) + 2e-3f : INFINITY;
 }
 
@@ -859,14 +869,14 @@ static_assert(sizeof(Counters) == TSDF_STATS_COPY_BYTES, "the header states the 
 static void fill_stats(const tsdf_volume* v, const Counters& h, tsdf_stats* o) {
     o->geo_updated = (int64_t)h.geo_updated;
     o->col_updated = (int64_t)h.col_updated;
-    o->geo_bricks = h.n_geo;
+    o->geo_bricks = (int64_t)h.n_geo + h.n_geo_open;
     o->col_bricks = h.n_col + h.n_col_light;
     o->visible_bricks = h.n_vis;
     o->total_bricks = (int64_t)v->nb[0] * v->nb[1] * v->nb[2];
     o->frames_counted = (int64_t)h.frames;
     o->total_geo_updated = (int64_t)(h.tot_geo_updated + h.geo_updated);
     o->total_col_updated = (int64_t)(h.tot_col_updated + h.col_updated);
-    o->total_geo_bricks = (int64_t)(h.tot_geo_bricks + h.n_geo);
+    o->total_geo_bricks = (int64_t)(h.tot_geo_bricks + h.n_geo + h.n_geo_open);
     o->total_col_bricks = (int64_t)(h.tot_col_bricks + h.n_col + h.n_col_light);
     o->total_visible_bricks = (int64_t)(h.tot_vis_bricks + h.n_vis);
     o->total_col_active_bricks = (int64_t)(h.tot_col_active + h.n_col_active);
@@ -921,7 +931,7 @@ tsdf_status tsdf_stats_collect(tsdf_volume* v, int32_t slot, tsdf_stats* o) {
         const Counters& g = v->stats_host[2 * slot + 1];
         h.n_geo = g.n_geo;
         h.n_vis = g.n_vis;
-        h.geo_next = g.geo_next;
+        h.n_geo_open = g.n_geo_open;
         h.n_geo_changed = g.n_geo_changed;
         h.geo_updated = g.geo_updated;
         h.frames = g.frames;
