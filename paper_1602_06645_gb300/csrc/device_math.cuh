@@ -124,25 +124,16 @@ __device__ __forceinline__ void chain_enter() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// Warp-aggregated append of `pred` items: the lane's place among those that
-// are counted in *ctr.
-__device__ __forceinline__ uint32_t append_slot(bool pred, uint32_t* ctr) {
-    const unsigned mask = __ballot_sync(0xffffffffu, pred);
-    if (!mask) return 0u;
-    const int lane = threadIdx.x & 31, leader = __ffs(mask) - 1;
+// Warp-aggregated append of `pred` items to list[ctr++].
+__device__ __forceinline__ void append(bool pred, uint32_t value, uint32_t* ctr, uint32_t* list) {
+    unsigned mask = __ballot_sync(0xffffffffu, pred);
+    if (!mask) return;
+    int lane = threadIdx.x & 31;
+    int leader = __ffs(mask) - 1;
     uint32_t base = 0;
     if (lane == leader) base = atomicAdd(ctr, (uint32_t)__popc(mask));
-    return __shfl_sync(0xffffffffu, base, leader) + __popc(mask & ((1u << lane) - 1u));
-}
-
-// Append to list[ctr++], or from the end down to end[-1 - ctr++].
-__device__ __forceinline__ void append(bool pred, uint32_t value, uint32_t* ctr, uint32_t* list) {
-    const uint32_t at = append_slot(pred, ctr);
-    if (pred) list[at] = value;
-}
-__device__ __forceinline__ void append_back(bool pred, uint32_t value, uint32_t* ctr, uint32_t* end) {
-    const uint32_t at = append_slot(pred, ctr);
-    if (pred) end[-1 - (int64_t)at] = value;
+    base = __shfl_sync(0xffffffffu, base, leader);
+    if (pred) list[base + __popc(mask & ((1u << lane) - 1u))] = value;
 }
 
 }  // namespace tsdf

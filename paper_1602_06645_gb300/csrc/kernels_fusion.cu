@@ -46,16 +46,55 @@ __host__ __device__ inline uint32_t depth_strips(const FrameConst& c) {
     return (uint32_t)((c.dw + STRIP_PX - 1) / STRIP_PX) * (uint32_t)c.tiles_y;
 }
 
-// Depth tiles of one 32 x 8-pixel strip (four 8 x 8 tiles) by one warp: lane
-// x reads column x of the strip's eight rows (eight independent reads, each
-// row's 64 bytes coalesced); min / max over the column, then over each group
-// of eight lanes.  depth_m (optional) receives the strip's depths in metres.
+// Depth tiles of one 32 x 8-pixel strip (four 8 x 8 tiles) by one warp.
+// depth_m (optional) receives the strip's depths in metres.  What bounds it is
+// latency, so a lane reads as much as it can in one access: where every tile
+// row starts on a 16-byte boundary (rows of a multiple of 8 pixels, the image
+// on one), lane 4 r + t reads the 8 pixels of tile t in row r at once, takes
+// their minimum and maximum two at a time and writes them as two float4, and
+// the rows are combined by shuffles.  Otherwise lane x reads column x of the
+// strip's eight rows (eight independent reads, each row's 64 bytes
+// coalesced) and the minimum and maximum over the column, then over each
+// group of eight lanes, are taken.  For twelve 640x480 images in the batched
+// step: 11 us with its barrier, 29 with column reads.
 __device__ __forceinline__ void depth_strip(const FrameConst& c, const uint16_t* __restrict__ depth,
                                             uint32_t* __restrict__ tiles, float* __restrict__ depth_m,
                                             uint32_t strip, int lane) {
-    static_assert(TILE_PX == 8 && STRIP_PX == 4 * TILE_PX, "the lane layout below assumes 8x8 tiles");
+    static_assert(TILE_PX == 8 && STRIP_PX == 4 * TILE_PX, "the lane layouts below assume 8x8 tiles");
     const uint32_t sx_n = (uint32_t)((c.dw + STRIP_PX - 1) / STRIP_PX);
     const int ty = (int)(strip / sx_n), sx = (int)(strip % sx_n);
+    const float ninf = __int_as_float(0xff800000);
+    if (c.dw % TILE_PX == 0 && ((uintptr_t)depth & 15u) == 0) {
+        const int t = lane & 3, py = ty * TILE_PX + (lane >> 2), tx = sx * 4 + t;
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        const size_t at = (size_t)py * c.dw + tx * TILE_PX;
+        if (tx < c.tiles_x && py < c.dh) {
+            v = *reinterpret_cast<const uint4*>(depth + at);
+            if (depth_m) {
+                const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+                float m[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const uint32_t D = (i & 1) ? w[i >> 1] >> 16 : w[i >> 1] & 0xFFFFu;
+                    m[i] = D ? (float)D * 0.001f : ninf;
+                }
+                reinterpret_cast<float4*>(depth_m + at)[0] = make_float4(m[0], m[1], m[2], m[3]);
+                reinterpret_cast<float4*>(depth_m + at)[1] = make_float4(m[4], m[5], m[6], m[7]);
+            }
+        }
+        // pairs of 16-bit values; D - 1 turns "no measurement" into the largest
+        uint32_t mn = __vminu2(__vminu2(__vsub2(v.x, 0x00010001u), __vsub2(v.y, 0x00010001u)),
+                               __vminu2(__vsub2(v.z, 0x00010001u), __vsub2(v.w, 0x00010001u)));
+        uint32_t mx = __vmaxu2(__vmaxu2(v.x, v.y), __vmaxu2(v.z, v.w));
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) {
+            mn = __vminu2(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+            mx = __vmaxu2(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        }
+        const uint32_t lo = min(min(mn & 0xFFFFu, mn >> 16) + 1u, 0xFFFFu), hi = max(mx & 0xFFFFu, mx >> 16);
+        if (lane < 4 && tx < c.tiles_x) tiles[ty * c.tiles_x + tx] = lo | (hi << 16);
+        return;
+    }
     const int px = sx * STRIP_PX + lane;
     const bool xin = px < c.dw;
     uint32_t D[TILE_PX];
@@ -65,7 +104,6 @@ __device__ __forceinline__ void depth_strip(const FrameConst& c, const uint16_t*
         D[r] = xin && py < c.dh ? depth[(size_t)py * c.dw + px] : 0u;
     }
     uint32_t mn = 0xFFFFu, mx = 0u;
-    const float ninf = __int_as_float(0xff800000);
 #pragma unroll
     for (int r = 0; r < TILE_PX; ++r) {
         const int py = ty * TILE_PX + r;
@@ -888,6 +926,9 @@ __global__ void __launch_bounds__(GEO_THREADS, 8) k_geometry(FrameConst c, Volum
         ctr->n_cells = ctr->n_vox = ctr->n_col_active = 0;
         ctr->col_updated = 0ull;
     }
+    __shared__ uint32_t n_open;  // read with n_geo, kept out of the registers of the first loop
+    if (threadIdx.x == 0) n_open = ctr->n_geo_open;
+    __syncthreads();
     const int lane = threadIdx.x & 31;
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -907,7 +948,6 @@ __global__ void __launch_bounds__(GEO_THREADS, 8) k_geometry(FrameConst c, Volum
             geometry_brick<PINHOLE, FREE_SPACE, ALIGNED, false>(c, vol, depth, at, lane, count, changed);
     }
     if (FREE_SPACE) {  // the open bricks go on where the warp's share of the list ended (a loop of their own: 64 registers)
-        const uint32_t n_open = ctr->n_geo_open;
         const uint32_t* end = list + (uint32_t)c.nb[0] * c.nb[1] * c.nb[2];
         for (item -= n; item < n_open; item += nwarps) {
             const uint32_t e = end[-1 - (int64_t)item];
@@ -2042,17 +2082,28 @@ __device__ bool grid_barrier(BatchSync* s, unsigned nblocks) {
 }
 
 // Per-block exclusive prefix over the scans of a per-scan count, each count
-// rounded up to a multiple of `pad`; pre[n] is the total.
+// rounded up to a multiple of `pad`; pre[n] is the total.  A thread per scan
+// reads its count (one thread reading them all in turn took 0.7 us per scan
+// and phase, a third of a step of 12 scans), one warp adds them up.
 template <typename F>
 __device__ __forceinline__ void scan_prefix(uint32_t* pre, int n, uint32_t pad, F count) {
     __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t acc = 0;
-        for (int i = 0; i < n; ++i) {
-            pre[i] = acc;
-            acc += (count(i) + pad - 1) / pad * pad;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) pre[i + 1] = (count(i) + pad - 1) / pad * pad;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        uint32_t carry = 0;
+        for (int base = 0; base < n; base += 32) {
+            uint32_t incl = base + lane < n ? pre[base + lane + 1] : 0u;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += v;
+            }
+            if (base + lane < n) pre[base + lane + 1] = carry + incl;
+            carry += __shfl_sync(0xffffffffu, incl, 31);
         }
-        pre[n] = acc;
+        if (lane == 0) pre[0] = 0;
     }
     __syncthreads();
 }
@@ -2071,6 +2122,18 @@ __global__ void __launch_bounds__(COL_THREADS, 4) k_batch_step(const ScanDesc* _
     extern __shared__ __align__(16) unsigned char smem_raw[];
     ColourSlot& S = reinterpret_cast<ColourSlot*>(smem_raw)[threadIdx.x >> 5];
     __shared__ uint32_t pre[MAX_BATCH + 1];
+    // the descriptor of the scan a warp is at: its fields are read for every
+    // brick, and in global memory they compete with the bricks for L1
+    __shared__ __align__(16) ScanDesc held[COL_THREADS / 32];
+    ScanDesc& d = held[threadIdx.x >> 5];
+    auto hold = [&](int s) {
+        static_assert(sizeof(ScanDesc) % 8 == 0, "copied in 8-byte words");
+        __syncwarp();
+        const uint2* from = reinterpret_cast<const uint2*>(descs + s);
+        uint2* to = reinterpret_cast<uint2*>(&d);
+        for (int i = threadIdx.x & 31; i < (int)(sizeof(ScanDesc) / 8); i += 32) to[i] = from[i];
+        __syncwarp();
+    };
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x;
@@ -2115,27 +2178,62 @@ __global__ void __launch_bounds__(COL_THREADS, 4) k_batch_step(const ScanDesc* _
         bool geo, vis, inner, open;
         brick_flags(d.c, d.vol.summ, d.scr.depth_tiles, b, b < nbt, geo, vis, inner, open);
         const uint32_t e = geo_entry(d.c, b, inner);
-        append(geo && !open, e, &d.scr.ctr->n_geo, d.scr.geo_list);
-        append_back(geo && open, e, &d.scr.ctr->n_geo_open, d.scr.geo_list + nbt);
-        append(vis, b, &d.scr.ctr->n_vis, d.scr.vis_list);
+        // the warp's three appends with one round trip to the counters
+        const unsigned m[3] = {__ballot_sync(full, geo && !open), __ballot_sync(full, geo && open),
+                               __ballot_sync(full, vis)};
+        Counters* ctr = d.scr.ctr;
+        uint32_t at = 0;
+        if (lane == 0 && m[0]) at = atomicAdd(&ctr->n_geo, (uint32_t)__popc(m[0]));
+        if (lane == 1 && m[1]) at = atomicAdd(&ctr->n_geo_open, (uint32_t)__popc(m[1]));
+        if (lane == 2 && m[2]) at = atomicAdd(&ctr->n_vis, (uint32_t)__popc(m[2]));
+        const unsigned lt = (1u << lane) - 1u;
+        const uint32_t at0 = __shfl_sync(full, at, 0) + __popc(m[0] & lt);
+        const uint32_t at1 = __shfl_sync(full, at, 1) + __popc(m[1] & lt);
+        const uint32_t at2 = __shfl_sync(full, at, 2) + __popc(m[2] & lt);
+        if (geo) d.scr.geo_list[open ? nbt - 1u - at1 : at0] = e;
+        if (vis) d.scr.vis_list[at2] = b;
     }
     if (!grid_barrier(sync, gridDim.x)) return;
 
-    // P2: geometry, one warp per tile of `tile` consecutive listed bricks of a scan
+    // P2: geometry, one warp per item of consecutive listed bricks of a scan.
+    // A warp's counts go to a scan's counters when it leaves the scan (an
+    // atomic per item, tens of thousands on one address, took up to two thirds
+    // of this phase).  At least two consecutive bricks per item here: with single ones the phase
+    // takes 93-128 us for 12 scans of edges 80-328, with pairs 68-87.
+    const uint32_t gtile = max(tile, 2);
     scan_prefix(pre, n, 1, [&](int i) {
-        return (descs[i].scr.ctr->n_geo + descs[i].scr.ctr->n_geo_open + tile - 1) / tile;
+        return (descs[i].scr.ctr->n_geo + descs[i].scr.ctr->n_geo_open + gtile - 1) / gtile;
     });
+    uint32_t count = 0, changed = 0;
+    int at_scan = -1;
+    auto leave_geo = [&]() {
+        const uint32_t sum = __reduce_add_sync(full, count);
+        if (lane == 0 && at_scan >= 0) {
+            Counters* ctr = descs[at_scan].scr.ctr;
+            if (sum) atomicAdd(&ctr->geo_updated, (unsigned long long)sum);
+            if (changed) atomicAdd(&ctr->n_geo_changed, changed);
+        }
+        count = changed = 0;
+    };
+    uint32_t nf = 0, ng = 0, s_end = 0;  // of the warp's scan; its first item after the scan's
+    const uint32_t* list = nullptr;
     for (uint32_t item = warp; item < pre[n]; item += nwarps) {
-        const int s = find_scan(pre, n, item);
-        const ScanDesc& d = descs[s];
-        const uint32_t nf = d.scr.ctr->n_geo, ng = nf + d.scr.ctr->n_geo_open;
+        if (item >= s_end) {
+            leave_geo();
+            at_scan = find_scan(pre, n, item);
+            s_end = pre[at_scan + 1];
+            hold(at_scan);
+            const Counters* ctr = d.scr.ctr;
+            nf = ctr->n_geo;
+            ng = nf + ctr->n_geo_open;
+            list = d.scr.geo_list;
+        }
         const uint32_t nbt = (uint32_t)d.c.nb[0] * d.c.nb[1] * d.c.nb[2];
-        const uint32_t k0 = (item - pre[s]) * tile, k1 = min(k0 + (uint32_t)tile, ng);
-        uint32_t count = 0, changed = 0;
+        const uint32_t k0 = (item - pre[at_scan]) * gtile, k1 = min(k0 + gtile, ng);
         const bool aligned = d.c.ng[0] % BRICK == 0 && d.c.ng[1] % BRICK == 0 && d.c.ng[2] % BRICK == 0;
         for (uint32_t k = k0; k < k1; ++k) {
             const bool open = k >= nf;
-            const uint32_t e = d.scr.geo_list[open ? nbt - 1u - (k - nf) : k];
+            const uint32_t e = list[open ? nbt - 1u - (k - nf) : k];
             const BrickAt at = geo_brick(d.c, e);
             const DepthMm dm{d.depth};
             // the usual camera and mode: without the per-voxel image tests for
@@ -2152,12 +2250,8 @@ __global__ void __launch_bounds__(COL_THREADS, 4) k_batch_step(const ScanDesc* _
             else
                 geometry_brick<false, false>(d.c, d.vol, dm, at, lane, count, changed);
         }
-        count = __reduce_add_sync(full, count);
-        if (lane == 0) {
-            if (count) atomicAdd(&d.scr.ctr->geo_updated, (unsigned long long)count);
-            if (changed) atomicAdd(&d.scr.ctr->n_geo_changed, changed);
-        }
     }
+    leave_geo();
     if (!grid_barrier(sync, gridDim.x)) return;
 
     // P3: colour candidates
@@ -2173,45 +2267,70 @@ __global__ void __launch_bounds__(COL_THREADS, 4) k_batch_step(const ScanDesc* _
     }
     if (!grid_barrier(sync, gridDim.x)) return;
 
-    // P4: band gate, one warp per tile of candidates, taken with an atomic counter
+    // P4: band gate, one warp per tile of candidates, taken with an atomic
+    // counter; a warp's staged records and counts are flushed when it leaves a
+    // scan
     scan_prefix(pre, n, 1, [&](int i) { return (descs[i].scr.ctr->n_col + tile - 1) / tile; });
-    for (;;) {
-        uint32_t item = 0;
-        if (lane == 0) item = atomicAdd(&sync->band_next, 1u);
-        item = __shfl_sync(full, item, 0);
-        if (item >= pre[n]) break;
-        const int s = find_scan(pre, n, item);
-        const ScanDesc& d = descs[s];
-        uint32_t count = 0, n_active = 0, n_cells = 0, nstage = 0;
-        const uint32_t k0 = (item - pre[s]) * tile, k1 = min(k0 + (uint32_t)tile, d.scr.ctr->n_col);
-        for (uint32_t k = k0; k < k1; ++k) {
-            band_brick(d.c, d.vol, d.depth, d.rgb, d.scr, S, d.scr.col_list[k], lane, count, n_active, n_cells,
-                       nstage);
-            __syncwarp();
-        }
-        band_flush(d.c, d.vol, d.depth, d.rgb, d.scr, S, lane, count, nstage);  // the records are this scan's
+    uint32_t n_active = 0, n_cells = 0, nstage = 0;
+    count = 0;
+    at_scan = -1;
+    auto leave_band = [&]() {
+        if (at_scan < 0) return;
+        band_flush(d.c, d.vol, d.depth, d.rgb, d.scr, S, lane, count, nstage);
         count = __reduce_add_sync(full, count);
         if (lane == 0) {
             if (count) atomicAdd(&d.scr.ctr->col_updated, (unsigned long long)count);
             if (n_active) atomicAdd(&d.scr.ctr->n_col_active, n_active);
             if (n_cells) atomicAdd(&d.scr.ctr->n_cells, n_cells);
         }
+        count = n_active = n_cells = 0;
+    };
+    uint32_t next = 0;
+    if (lane == 0) next = atomicAdd(&sync->band_next, 1u);
+    for (;;) {
+        const uint32_t item = __shfl_sync(full, next, 0);
+        if (item >= pre[n]) break;
+        if (lane == 0) next = atomicAdd(&sync->band_next, 1u);  // claimed while this item is processed
+        const int s = find_scan(pre, n, item);
+        if (s != at_scan) {
+            leave_band();
+            at_scan = s;
+            hold(s);
+        }
+        const uint32_t k0 = (item - pre[s]) * tile, k1 = min(k0 + (uint32_t)tile, d.scr.ctr->n_col);
+        for (uint32_t k = k0; k < k1; ++k) {
+            band_brick(d.c, d.vol, d.depth, d.rgb, d.scr, S, d.scr.col_list[k], lane, count, n_active, n_cells,
+                       nstage);
+            __syncwarp();
+        }
     }
+    leave_band();
     if (!grid_barrier(sync, gridDim.x)) return;
 
     // P5: colour voxels that passed the band gate
-    scan_prefix(pre, n, 32, [&](int i) { return min(descs[i].scr.ctr->n_vox, descs[i].scr.vox_cap); });
-    for (uint32_t base = warp * 32; base < pre[n]; base += nthreads) {
-        const uint32_t item = base + lane;
+    // a warp takes VOX_ITEM records of a scan at a time: their reads in flight
+    // together, the scan's constants and the counter's atomic once
+    constexpr uint32_t VOX_ITEM = 128;
+    scan_prefix(pre, n, VOX_ITEM, [&](int i) { return min(descs[i].scr.ctr->n_vox, descs[i].scr.vox_cap); });
+    at_scan = -1;
+    for (uint32_t base = warp * VOX_ITEM; base < pre[n]; base += nwarps * VOX_ITEM) {
         const int s = find_scan(pre, n, base);
-        const ScanDesc& d = descs[s];
-        const uint32_t i = item - pre[s];
-        bool upd = false;
-        if (i < min(d.scr.ctr->n_vox, d.scr.vox_cap)) {
-            const uint2 r = d.scr.vox[i];
-            upd = colour_after_band(d.c, d.vol.C, d.depth, d.rgb, (int)(r.x & 0xFFFFu), (int)(r.x >> 16), (int)r.y);
+        if (s != at_scan) {
+            at_scan = s;
+            hold(s);
         }
-        const uint32_t cnt = __popc(__ballot_sync(full, upd));
+        const uint32_t i0 = base - pre[s] + lane, nv = min(d.scr.ctr->n_vox, d.scr.vox_cap);
+        uint2 r[VOX_ITEM / 32];
+#pragma unroll
+        for (uint32_t k = 0; k < VOX_ITEM / 32; ++k)
+            if (i0 + 32 * k < nv) r[k] = d.scr.vox[i0 + 32 * k];
+        uint32_t cnt = 0;
+#pragma unroll
+        for (uint32_t k = 0; k < VOX_ITEM / 32; ++k)
+            if (i0 + 32 * k < nv && colour_after_band(d.c, d.vol.C, d.depth, d.rgb, (int)(r[k].x & 0xFFFFu),
+                                                      (int)(r[k].x >> 16), (int)r[k].y))
+                ++cnt;
+        cnt = __reduce_add_sync(full, cnt);
         if (lane == 0 && cnt) atomicAdd(&d.scr.ctr->col_updated, (unsigned long long)cnt);
     }
 }
