@@ -102,7 +102,7 @@ struct AdjBuffers {
     uint32_t slot_cap;
     int32_t max_frames;
     AdjFrame* frames;
-    uint32_t* counters;     // [0] pairs, [1] slots
+    uint32_t* counters;     // [0] pairs, [1] slots, [2] finalize errors, [3] finished blocks of a backward pass (0 between passes)
     double* partials;       // per-block gradient partials (10 each)
     double* grad;           // 10 reduced gradient entries
 };

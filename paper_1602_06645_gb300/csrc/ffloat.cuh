@@ -62,4 +62,35 @@ __device__ __forceinline__ ff ff_div(ff a, ff b) {
     return fast_two_sum(q, __fdiv_rn(r.hi, b.hi));
 }
 
+// A sum of binary32 terms as three binary32 numbers: the running sum, the sum
+// of its rounding errors, and the sum of that sum's.  Both additions are
+// error-free (TwoSum), so only the third component rounds: the total carries
+// about 70 bits, more than a binary64 sum of the same terms, without the
+// binary64 pipe (some 64 cycles per warp instruction on this GPU).
+struct fsum3 {
+    float hi, mid, lo;
+};
+
+__device__ __forceinline__ void fsum3_add(fsum3& s, float x) {
+    const ff a = two_sum(s.hi, x), b = two_sum(s.mid, a.lo);
+    s.hi = a.hi;
+    s.mid = b.hi;
+    s.lo += b.lo;
+}
+
+__device__ __forceinline__ fsum3 fsum3_merge(const fsum3& s, const fsum3& t) {
+    const ff a = two_sum(s.hi, t.hi), b = two_sum(s.mid, t.mid), c = two_sum(b.hi, a.lo);
+    return {a.hi, c.hi, (s.lo + t.lo) + (b.lo + c.lo)};
+}
+
+// (An infinite or NaN running sum is the sum: its rounding errors are then NaN.)
+__device__ __forceinline__ double fsum3_value(const fsum3& s) {
+    return isfinite(s.hi) ? (double)s.hi + ((double)s.mid + (double)s.lo) : (double)s.hi;
+}
+
+__device__ __forceinline__ fsum3 fsum3_shfl_xor(const fsum3& s, int lanes) {
+    return {__shfl_xor_sync(0xffffffffu, s.hi, lanes), __shfl_xor_sync(0xffffffffu, s.mid, lanes),
+            __shfl_xor_sync(0xffffffffu, s.lo, lanes)};
+}
+
 }  // namespace tsdf
