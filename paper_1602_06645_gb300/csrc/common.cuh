@@ -292,8 +292,11 @@ struct RayConst {
 cudaError_t launch_ray_map(const BrickSummary* summ, const int32_t nb[3], bool plain_f, uint16_t* map,
                            cudaStream_t stream);
 // Reads the map of the volume as it is (launch_ray_map after its last change).
+// behind: the launch before this one on the stream is another ray cast of the
+// same volume, beside which this one may run.
 cudaError_t launch_raycast(const RayConst& c, const float* F, const uint8_t* W, const uint32_t* C, const uint16_t* map,
-                           float* range, float* vertex, float* normal, uint32_t* rgbw, cudaStream_t stream);
+                           float* range, float* vertex, float* normal, uint32_t* rgbw, bool behind,
+                           cudaStream_t stream);
 
 // ------------------------------------------------------- camera tracking --
 // One pyramid level of one tracking step (see tsdf_track in tsdf.h).

@@ -78,6 +78,14 @@ __device__ __forceinline__ void fsum3_add(fsum3& s, float x) {
     s.lo += b.lo;
 }
 
+// Adds x y, whose rounding error one fused multiply-add gives exactly.
+__device__ __forceinline__ void fsum3_add_product(fsum3& s, float x, float y) {
+    const ff p = two_prod(x, y), a = two_sum(s.hi, p.hi), b = two_sum(s.mid, p.lo), c = two_sum(b.hi, a.lo);
+    s.hi = a.hi;
+    s.mid = c.hi;
+    s.lo += b.lo + c.lo;
+}
+
 __device__ __forceinline__ fsum3 fsum3_merge(const fsum3& s, const fsum3& t) {
     const ff a = two_sum(s.hi, t.hi), b = two_sum(s.mid, t.mid), c = two_sum(b.hi, a.lo);
     return {a.hi, c.hi, (s.lo + t.lo) + (b.lo + c.lo)};

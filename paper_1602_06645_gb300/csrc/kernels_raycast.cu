@@ -24,7 +24,8 @@
 // Measured (24 frames around a scene of 20 primitives, 2 m cube): 640x480 rays
 // through 512^3, 1064 -> 256 us and 5 us for the map; 1920x1080 through 192^3,
 // 1936 -> 689 us and 3 us; the three prediction levels of a tracked frame at
-// 512^3, 2454 -> 613 us.
+// 512^3, 2454 -> 613 us one after another, about 430 us beside one another
+// (launch_raycast, behind).  Eight blocks per SM; 7, 10 and 12 were slower.
 #include <cfloat>
 #include <cstdint>
 
@@ -226,15 +227,22 @@ __device__ __forceinline__ bool rc_pair(const RayConst& c, const float* __restri
     return true;
 }
 
-__global__ void __launch_bounds__(RC_THREADS) k_raycast(RayConst c, const float* __restrict__ F,
+__global__ void __launch_bounds__(RC_THREADS, 8) k_raycast(RayConst c, const float* __restrict__ F,
                                                         const uint8_t* __restrict__ W, const uint32_t* __restrict__ C,
                                                         const uint16_t* __restrict__ map, float* __restrict__ range,
                                                         float* __restrict__ vertex, float* __restrict__ normal,
                                                         uint32_t* __restrict__ rgbw) {
+    // Casts launched as a chain (launch_raycast, behind) read nothing of one
+    // another: the next one's blocks may start at once, filling the SMs this
+    // one's last rays leave; each ends after the one before it.
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int x = blockIdx.x * RC_BX + (warp & 1) * 8 + (lane & 7);
     const int y = blockIdx.y * RC_BY + (warp >> 1) * 4 + (lane >> 3);
-    if (x >= c.width || y >= c.height) return;
+    if (x >= c.width || y >= c.height) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        return;
+    }
     const float fx = (float)x, fy = (float)y;
     const float dc0 = fmaf(c.Kinv[0], fx, fmaf(c.Kinv[1], fy, c.Kinv[2]));
     const float dc1 = fmaf(c.Kinv[3], fx, fmaf(c.Kinv[4], fy, c.Kinv[5]));
@@ -412,6 +420,7 @@ __global__ void __launch_bounds__(RC_THREADS) k_raycast(RayConst c, const float*
         normal[3 * i + 2] = n[2];
     }
     if (rgbw) rgbw[i] = col;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 }  // namespace
@@ -425,10 +434,18 @@ cudaError_t launch_ray_map(const BrickSummary* summ, const int32_t nb[3], bool p
 }
 
 cudaError_t launch_raycast(const RayConst& c, const float* F, const uint8_t* W, const uint32_t* C, const uint16_t* map,
-                           float* range, float* vertex, float* normal, uint32_t* rgbw, cudaStream_t stream) {
-    const dim3 grid((c.width + RC_BX - 1) / RC_BX, (c.height + RC_BY - 1) / RC_BY);
-    k_raycast<<<grid, RC_THREADS, 0, stream>>>(c, F, W, C, map, range, vertex, normal, rgbw);
-    return cudaGetLastError();
+                           float* range, float* vertex, float* normal, uint32_t* rgbw, bool behind,
+                           cudaStream_t stream) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((c.width + RC_BX - 1) / RC_BX, (c.height + RC_BY - 1) / RC_BY);
+    cfg.blockDim = dim3(RC_THREADS);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = behind ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k_raycast, c, F, W, C, map, range, vertex, normal, rgbw);
 }
 
 }  // namespace tsdf

@@ -9,6 +9,7 @@
 #include <cstdint>
 
 #include "common.cuh"
+#include "ffloat.cuh"
 
 namespace tsdf {
 namespace {
@@ -97,34 +98,36 @@ __device__ __forceinline__ void rigid3(const float* R, const float* t, float x, 
 
 // What bounds a step is the binary64 pipe, which takes about 64 cycles per
 // warp instruction on each quarter of an SM whatever the number of active
-// lanes, so both parts are written for few binary64 instructions per warp:
-//  * terms: the products of two binary32 factors are exact in binary64, so
-//    one fused multiply-add per sum rounds as a product and a sum would;
-//    the count is an integer; the 28 sums of a warp's lanes are reduced by
-//    halves (each exchange halves the sums a lane holds: 31 additions instead
-//    of 5 per sum, 145), the warps' and blocks' sums with one lane per sum;
+// lanes, so both parts keep off it where they can:
+//  * terms: the 28 sums of products are kept per thread as error-free triples
+//    of binary32 numbers (fsum3: 22 instructions per product, more bits than
+//    a binary64 sum), the count as an integer; the sums of a warp's lanes are
+//    reduced by halves (each exchange halves the sums a lane holds: 31
+//    additions instead of 5 per sum, 145) and turned into binary64 one per
+//    lane, the warps' and blocks' sums added with one lane per sum;
 //  * solve: by the last block to finish, one warp, a lane per row or matrix
 //    entry (one thread alone took 28 us per step).
 // One launch per step; its blocks start while the previous step finishes and
 // read their first pixels before waiting for that step's pose.
-// Measured per step: 27.6 us at 640x480, 19.2 at 320x240, 16.8 at 160x120
-// (about 17 us of each is the fixed chain of wait, reduction and solve);
-// separate kernels for the terms and a one-thread solve took 57 us on average
-// over a frame's 19 steps.
+// Measured per step: 24.0 us at 640x480, 17.8 at 320x240, 14.2 at 160x120
+// (some 14 us of each is the fixed chain of wait, reduction and solve); with
+// the sums in binary64, one fused multiply-add per product, 27.6, 19.2 and
+// 16.8 us; with separate kernels for the terms and a one-thread solve 57 us on
+// average over a frame's 19 steps.
 constexpr int NSLOT = 32;  // the 29 sums, padded
 
-// Sums of a warp's lanes: on return lane l holds the sum of v[l].
-__device__ __forceinline__ double warp_sums(double (&v)[NSLOT], int lane) {
+// Sums of a warp's lanes: lane l gets the sum of v[l].
+__device__ __forceinline__ double warp_sums(fsum3 (&v)[NSLOT], int lane) {
 #pragma unroll
     for (int h = NSLOT / 2; h >= 1; h >>= 1) {
         const bool up = (lane & h) != 0;
 #pragma unroll
         for (int k = 0; k < h; ++k) {
-            const double give = up ? v[k] : v[k + h], keep = up ? v[k + h] : v[k];
-            v[k] = keep + __shfl_xor_sync(0xffffffffu, give, h);
+            const fsum3 give = up ? v[k] : v[k + h], keep = up ? v[k + h] : v[k];
+            v[k] = fsum3_merge(keep, fsum3_shfl_xor(give, h));
         }
     }
-    return v[0];
+    return fsum3_value(v[0]);
 }
 
 // exp coefficients of a rotation by angle a: row 0 sin(a)/a, row 1
@@ -272,9 +275,9 @@ __global__ void __launch_bounds__(TRACK_THREADS) k_icp_step(TrackLevel L, double
         for (int k = 0; k < 3; ++k) R[r * 3 + k] = (float)pose[r * 4 + k];
         t[r] = (float)pose[r * 4 + 3];
     }
-    double acc[NSLOT];
+    fsum3 acc[NSLOT];
 #pragma unroll
-    for (int k = 0; k < NSLOT; ++k) acc[k] = 0.0;
+    for (int k = 0; k < NSLOT; ++k) acc[k] = {0.0f, 0.0f, 0.0f};
     unsigned pairs = 0;
     for (; i < npx; i += gridDim.x * blockDim.x) {
         const float v0 = vx, v1 = vy, v2 = vz, m0 = nx, m1 = ny, m2 = nz;
@@ -300,16 +303,14 @@ __global__ void __launch_bounds__(TRACK_THREADS) k_icp_step(TrackLevel L, double
         if (fmaf(e0, e0, fmaf(e1, e1, e2 * e2)) > L.max_dist2) continue;
         if (!(fmaf(m[0], n0, fmaf(m[1], n1, m[2] * n2)) >= L.min_cos)) continue;
         const float r = fmaf(e0, n0, fmaf(e1, n1, e2 * n2));
-        // J and r; the products of two of them are exact in binary64
-        const double J[7] = {n0, n1, n2, (double)(p[1] * n2 - p[2] * n1), (double)(p[2] * n0 - p[0] * n2),
-                             (double)(p[0] * n1 - p[1] * n0), (double)r};
+        const float J[7] = {n0, n1, n2, p[1] * n2 - p[2] * n1, p[2] * n0 - p[0] * n2, p[0] * n1 - p[1] * n0, r};
         int k = 0;
 #pragma unroll
         for (int a = 0; a < 6; ++a)
 #pragma unroll
-            for (int b = a; b < 6; ++b, ++k) acc[k] = __fma_rn(J[a], J[b], acc[k]);
+            for (int b = a; b < 6; ++b, ++k) fsum3_add_product(acc[k], J[a], J[b]);
 #pragma unroll
-        for (int a = 0; a < 7; ++a) acc[21 + a] = __fma_rn(J[a], J[6], acc[21 + a]);
+        for (int a = 0; a < 7; ++a) fsum3_add_product(acc[21 + a], J[a], J[6]);
         ++pairs;
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;

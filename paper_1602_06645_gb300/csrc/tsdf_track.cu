@@ -122,9 +122,7 @@ extern "C" tsdf_status tsdf_track(tsdf_volume* v, const uint16_t* depth_mm, tsdf
     if (e == cudaSuccess) e = cudaMemcpyAsync(pose, T_init, 16 * sizeof(double), cudaMemcpyHostToDevice, v->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(finished, 0, sizeof *finished, v->stream);
     if (e == cudaSuccess) e = tsdf::launch_track_pyramid(d_depth, W, H, p.levels, dl, v->stream);
-    if (e == cudaSuccess) e = tsdf::launch_ray_map(v->vol.summ, v->nb, v->plain_f, v->scr.ray_map, v->stream);
     if (e != cudaSuccess) return cuda_fail(v, e, "track: pyramid");
-
     // world -> prediction camera, as the fusion's frame constants invert a pose
     tsdf::TrackLevel L;
     std::memset(&L, 0, sizeof L);
@@ -139,12 +137,14 @@ extern "C" tsdf_status tsdf_track(tsdf_volume* v, const uint16_t* depth_mm, tsdf
     L.max_dist2 = p.max_distance * p.max_distance;
     L.min_cos = p.min_normal_cos;
     tsdf_raycast_params rp = {p.near_m, p.far_m, 0.0f, 0.0f};
-    int step = 0;
-    int step_level[TSDF_TRACK_MAX_STEPS];
-    for (int l = p.levels - 1; l >= 0; --l) {
-        const int w = W >> l, h = H >> l;
+    // the maps of every level, then the predictions, the largest first (they
+    // run beside one another), then the steps from the coarsest level on
+    tsdf::RayConst rc[TSDF_TRACK_MAX_LEVELS];
+    float Kls[TSDF_TRACK_MAX_LEVELS][9];
+    for (int l = 0; l < p.levels; ++l) {
         const double s = std::ldexp(1.0, -l);
-        float Kl[9] = {0.0f};
+        float* Kl = Kls[l];
+        std::memset(Kl, 0, sizeof Kls[l]);
         Kl[0] = (float)((double)K_depth[0] * s);
         Kl[4] = (float)((double)K_depth[4] * s);
         Kl[2] = (float)(((double)K_depth[2] + 0.5) * s - 0.5);
@@ -152,17 +152,22 @@ extern "C" tsdf_status tsdf_track(tsdf_volume* v, const uint16_t* depth_mm, tsdf
         Kl[8] = 1.0f;
         const float kinv4[4] = {(float)(1.0 / (double)Kl[0]), (float)(1.0 / (double)Kl[4]),
                                 (float)(-(double)Kl[2] / (double)Kl[0]), (float)(-(double)Kl[5] / (double)Kl[4])};
-        e = tsdf::launch_track_maps(dl[l], w, h, kinv4, Vl[l], Nl[l], v->stream);
+        e = tsdf::launch_track_maps(dl[l], W >> l, H >> l, kinv4, Vl[l], Nl[l], v->stream);
         if (e != cudaSuccess) return cuda_fail(v, e, "track: maps");
-        tsdf::RayConst rc;
-        const tsdf_status rs = raycast_constants(v, Kl, T_world_depth_prev, tsdf_image_size{w, h}, &rp, rc);
+        const tsdf_status rs = raycast_constants(v, Kl, T_world_depth_prev, tsdf_image_size{W >> l, H >> l}, &rp, rc[l]);
         if (rs != TSDF_OK) return rs;
-        e = tsdf::launch_raycast(rc, v->vol.F, v->vol.W, v->vol.C, v->scr.ray_map, nullptr, PVl[l], PNl[l], nullptr,
-                                 v->stream);
-        if (e != cudaSuccess) return cuda_fail(v, e, "track: prediction");
-        L.w = w;
-        L.h = h;
-        std::memcpy(L.K, Kl, sizeof Kl);
+    }
+    e = tsdf::launch_ray_map(v->vol.summ, v->nb, v->plain_f, v->scr.ray_map, v->stream);
+    for (int l = 0; l < p.levels && e == cudaSuccess; ++l)
+        e = tsdf::launch_raycast(rc[l], v->vol.F, v->vol.W, v->vol.C, v->scr.ray_map, nullptr, PVl[l], PNl[l], nullptr,
+                                 l > 0, v->stream);
+    if (e != cudaSuccess) return cuda_fail(v, e, "track: prediction");
+    int step = 0;
+    int step_level[TSDF_TRACK_MAX_STEPS];
+    for (int l = p.levels - 1; l >= 0; --l) {
+        L.w = W >> l;
+        L.h = H >> l;
+        std::memcpy(L.K, Kls[l], sizeof Kls[l]);
         L.V = Vl[l];
         L.N = Nl[l];
         L.PV = PVl[l];
