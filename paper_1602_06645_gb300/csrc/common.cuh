@@ -327,15 +327,18 @@ struct MeshConst {
     float s_g;
     float origin[3];
 };
+// Marching-cubes case table: entry m, for the mask m of inside corners, holds
+// the triangle count and then three cell-edge numbers per triangle.  Passed as
+// a kernel parameter (4 KB).
+struct CubeCases {
+    alignas(16) uint8_t t[256][16];
+};
 // Candidate bricks (cells whose corners can have both signs), then one warp per
 // candidate; triangles are appended at *count (slots beyond cap are counted,
 // not written).
 cudaError_t launch_mesh(const MeshConst& c, const float* F, const uint8_t* W, const BrickSummary* summ,
                         uint32_t* list, uint32_t* n_list, float* out, uint64_t cap, unsigned long long* count,
-                        bool cubes, cudaStream_t stream);
-// Copy the 256-entry marching-cubes case table (count, then edge triples) to
-// the device.
-cudaError_t upload_cube_cases(const uint8_t (*table)[16], cudaStream_t stream);
+                        bool cubes, const CubeCases& cases, cudaStream_t stream);
 // Colour volume for texture maps (see tsdf_texture_fill in tsdf.h).
 struct ColourConst {
     int32_t nc[3], ncb[3];

@@ -15,7 +15,7 @@ namespace {
 constexpr int MESH_THREADS = 128;  // 4 warps, one candidate brick per warp
 constexpr int TILE_M = BRICK + 1;  // cells of a brick need one more voxel on the + sides
 constexpr int TILE_M3 = TILE_M * TILE_M * TILE_M;
-constexpr int CASE_BYTES = 16;     // a row of the marching-cubes case table
+constexpr int CASE_BYTES = 16;     // a row of the marching-cubes case table (CubeCases)
 
 // Corner orders of the six tetrahedra of a cell (main-diagonal split): for the
 // axis orderings (x,y,z), (x,z,y), (y,x,z), (y,z,x), (z,x,y), (z,y,x) the path
@@ -28,11 +28,6 @@ __device__ __forceinline__ void tet_corners(int t, int c[4]) {
     c[2] = c[1] | (1 << a1);
     c[3] = 7;
 }
-
-// Marching-cubes case table (built on the host from the rules in tsdf.h):
-// entry m, for the mask m of inside corners, holds the triangle count and
-// then three cell-edge numbers per triangle.
-__constant__ __align__(16) uint8_t c_cube_cases[256][CASE_BYTES];
 
 // Lower and upper corner of cell edge e = 4 a + r: the lower corner is r with
 // a zero bit inserted at position a.
@@ -184,9 +179,10 @@ __device__ void cube_emit(const MeshConst& c, const int base[3], const float Fc[
 }
 
 // Stage one tile voxel.
+template <bool KEEP_F>
 __device__ __forceinline__ void mesh_stage(MeshSlot& S, int tx, int ty, int tz, float f, bool observed) {
     const int r = tz * TILE_M + ty;
-    S.F[r * TILE_M + tx] = f;
+    if (KEEP_F) S.F[r * TILE_M + tx] = f;
     const uint32_t bits = (observed ? 1u : 0u) | (f < 0.0f ? 1u << 9 : 0u);
     if (bits) atomicOr(&S.row[r], bits << tx);
 }
@@ -206,20 +202,22 @@ __device__ __forceinline__ uint32_t cell_mask(const MeshSlot& S, int cx, int cy,
 // triangles' places with one atomic per brick (one per 32 cells, some 130,000
 // on one address, bounded the kernel), and where nothing is written (cap 0)
 // with one per block.  Counting and then writing the triangles of the fused
-// 512^3 scan (24 frames, about 700,000): 2 x 169 -> 131 us together.
-template <bool CUBES>
-__global__ void __launch_bounds__(MESH_THREADS) k_mesh(MeshConst c, const float* __restrict__ F,
+// 512^3 scan (24 frames, about 700,000): 2 x 169 -> 32 + 95 us.
+// WRITE: false only counts (cap is 0), without keeping the F of the tile.
+template <bool CUBES, bool WRITE>
+__global__ void __launch_bounds__(MESH_THREADS) k_mesh(const __grid_constant__ CubeCases table, MeshConst c,
+                                                      const float* __restrict__ F,
                                                       const uint8_t* __restrict__ W,
                                                       const uint32_t* __restrict__ list,
                                                       const uint32_t* __restrict__ n_list, float* __restrict__ out,
                                                       uint64_t cap, unsigned long long* __restrict__ count) {
     __shared__ MeshSlot slots[MESH_THREADS / 32];
-    // the case table: lanes look up different rows, which constant memory would serve one by one
+    // the case table: lanes look up different rows, which the parameter space would serve one by one
     __shared__ __align__(16) uint8_t cases[CUBES ? 256 * CASE_BYTES : 16];
     __shared__ unsigned long long block_total;
     if (CUBES) {
         for (int i = threadIdx.x; i < 256; i += MESH_THREADS)
-            reinterpret_cast<uint4*>(cases)[i] = reinterpret_cast<const uint4*>(c_cube_cases)[i];
+            reinterpret_cast<uint4*>(cases)[i] = reinterpret_cast<const uint4*>(table.t)[i];
     }
     if (threadIdx.x == 0) block_total = 0ull;
     __syncthreads();
@@ -280,7 +278,7 @@ __global__ void __launch_bounds__(MESH_THREADS) k_mesh(MeshConst c, const float*
             uint32_t bits = 0;
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                S.F[r * TILE_M + x0 + i] = fv[i];
+                if (WRITE) S.F[r * TILE_M + x0 + i] = fv[i];
                 const bool seen = yz && base0[0] + x0 + i < c.ng[0] && ((w[j] >> (8 * i)) & 0xFFu) != 0u;
                 bits |= ((seen ? 1u : 0u) | (fv[i] < 0.0f ? 1u << 9 : 0u)) << i;
             }
@@ -288,7 +286,7 @@ __global__ void __launch_bounds__(MESH_THREADS) k_mesh(MeshConst c, const float*
         }
 #pragma unroll
         for (int i = 0; i < 7; ++i)
-            if (i < 6 || lane < 25) mesh_stage(S, hx[i], hy[i], hz[i], hf[i], ho[i]);
+            if (i < 6 || lane < 25) mesh_stage<WRITE>(S, hx[i], hy[i], hz[i], hf[i], ho[i]);
         __syncwarp();
         // the crossed cells of two cell rows (y, z) per lane, compacted
         uint32_t act[2];
@@ -324,7 +322,7 @@ __global__ void __launch_bounds__(MESH_THREADS) k_mesh(MeshConst c, const float*
         int cell;
         for (int k = lane; k < nact; k += 32) total += triangles(k, m, cell);
         total = __reduce_add_sync(full, total);
-        if (cap == 0) {
+        if (!WRITE) {
             counted += total;
             __syncwarp();
             continue;
@@ -354,7 +352,7 @@ __global__ void __launch_bounds__(MESH_THREADS) k_mesh(MeshConst c, const float*
         }
         __syncwarp();
     }
-    if (cap == 0) {
+    if (!WRITE) {
         if (lane == 0 && counted) atomicAdd(&block_total, counted);
         __syncthreads();
         if (threadIdx.x == 0 && block_total) atomicAdd(count, block_total);
@@ -625,27 +623,18 @@ __global__ void __launch_bounds__(256) k_tex_fill(ColourConst c, const uint32_t*
 
 }  // namespace
 
-cudaError_t upload_cube_cases(const uint8_t (*table)[16], cudaStream_t stream) {
-    return cudaMemcpyToSymbolAsync(c_cube_cases, table, sizeof(c_cube_cases), 0, cudaMemcpyHostToDevice, stream);
-}
-
 cudaError_t launch_mesh(const MeshConst& c, const float* F, const uint8_t* W, const BrickSummary* summ,
                         uint32_t* list, uint32_t* n_list, float* out, uint64_t cap, unsigned long long* count,
-                        bool cubes, cudaStream_t stream) {
+                        bool cubes, const CubeCases& cases, cudaStream_t stream) {
     const uint32_t nbt = (uint32_t)c.nb[0] * c.nb[1] * c.nb[2];
     k_mesh_bricks<<<(nbt + 255) / 256, 256, 0, stream>>>(c, summ, list, n_list);
     int sms = 0, dev = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (cubes) {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mesh<true>, MESH_THREADS, 0);
-        k_mesh<true><<<max(1, sms * max(1, per_sm)), MESH_THREADS, 0, stream>>>(c, F, W, list, n_list, out, cap,
-                                                                               count);
-    } else {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mesh<false>, MESH_THREADS, 0);
-        k_mesh<false><<<max(1, sms * max(1, per_sm)), MESH_THREADS, 0, stream>>>(c, F, W, list, n_list, out, cap,
-                                                                                count);
-    }
+    auto k = cubes ? (cap ? k_mesh<true, true> : k_mesh<true, false>)
+                   : (cap ? k_mesh<false, true> : k_mesh<false, false>);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, MESH_THREADS, 0);
+    k<<<max(1, sms * max(1, per_sm)), MESH_THREADS, 0, stream>>>(cases, c, F, W, list, n_list, out, cap, count);
     return cudaGetLastError();
 }
 

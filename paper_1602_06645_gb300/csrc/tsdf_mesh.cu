@@ -62,9 +62,7 @@ tsdf::MeshConst mesh_const(const tsdf_volume* v) {
 // The 256-case table of tsdf.h's marching-cubes rules, built once.  Corner k
 // sits at (k & 1, (k >> 1) & 1, k >> 2); edge 4 a + r joins the r-th corner
 // with bit a clear (in increasing order) to its neighbour along a.
-struct CubeCases {
-    uint8_t t[256][16];  // triangle count, then edge triples
-};
+using tsdf::CubeCases;
 
 int cube_edge(int p, int q) {
     const int lo = std::min(p, q), a = (p ^ q) == 1 ? 0 : ((p ^ q) == 2 ? 1 : 2);
@@ -171,23 +169,23 @@ extern "C" tsdf_status tsdf_mesh_ex(tsdf_volume* v, int32_t method, float* trian
         return fail(v, TSDF_ERR_INVALID_ARG, "mesh: need n_triangles, capacity >= 0 and a buffer for it");
     Temps t(v);
     const size_t nbt = (size_t)v->nb[0] * v->nb[1] * v->nb[2];
-    uint32_t* list = (uint32_t*)t.get(nbt * sizeof(uint32_t));
-    uint32_t* n_list = (uint32_t*)t.get(sizeof(uint32_t) + sizeof(unsigned long long) * 2);
+    // one allocation: the counters (list length, triangles), then the brick list
+    uint32_t* n_list = (uint32_t*)t.get(16 + nbt * sizeof(uint32_t));
     const size_t out_bytes = (size_t)capacity * 9 * sizeof(float);
     float* out = (float*)output(t, triangles, out_bytes);
-    if (!list || !n_list || (capacity > 0 && !out)) return fail(v, TSDF_ERR_OOM, "mesh: scratch buffers");
+    if (!n_list || (capacity > 0 && !out)) return fail(v, TSDF_ERR_OOM, "mesh: scratch buffers");
     unsigned long long* count = reinterpret_cast<unsigned long long*>(n_list + 2);
-    cudaError_t e = cudaMemsetAsync(n_list, 0, sizeof(uint32_t) + sizeof(unsigned long long) * 2, v->stream);
-    if (e == cudaSuccess && method == TSDF_MESH_CUBES) e = tsdf::upload_cube_cases(cube_cases().t, v->stream);
+    cudaError_t e = cudaMemsetAsync(n_list, 0, 16, v->stream);
     if (e == cudaSuccess)
-        e = tsdf::launch_mesh(mesh_const(v), v->vol.F, v->vol.W, v->vol.summ, list, n_list, out,
-                              (uint64_t)capacity, count, method == TSDF_MESH_CUBES, v->stream);
+        e = tsdf::launch_mesh(mesh_const(v), v->vol.F, v->vol.W, v->vol.summ, n_list + 4, n_list, out,
+                              (uint64_t)capacity, count, method == TSDF_MESH_CUBES, cube_cases(), v->stream);
     unsigned long long total = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&total, count, sizeof total, cudaMemcpyDeviceToHost, v->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(v->stream);
-    if (e == cudaSuccess)
+    if (e == cudaSuccess && out != triangles) {
         e = finish(v, triangles, out, (size_t)std::min<int64_t>(capacity, (int64_t)total) * 9 * sizeof(float));
-    if (e == cudaSuccess) e = cudaStreamSynchronize(v->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(v->stream);
+    }
     if (e != cudaSuccess) return cuda_fail(v, e, "mesh");
     *n_triangles = (int64_t)total;
     return TSDF_OK;
