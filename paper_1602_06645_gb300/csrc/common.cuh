@@ -192,7 +192,7 @@ cudaError_t launch_frame_post(const FrameConst& c, const Volumes& v, const Scrat
 cudaError_t launch_frame(const FrameConst& c, const Volumes& v, const Scratch& s, const uint16_t* depth,
                          const uint8_t* rgb, const LaunchGrids& g, cudaStream_t stream, cudaEvent_t* ev = nullptr);
 int geometry_blocks_per_sm();
-int geometry_linear_blocks_per_sm();  // k_geometry_linear (the allocation-free entry point)
+int geometry_linear_blocks_per_sm();  // the linear-volume kernels (the allocation-free entry point)
 int colour_blocks_per_sm();
 int voxel_blocks_per_sm();
 int fused_blocks_per_sm();
@@ -292,10 +292,12 @@ struct RayConst {
 cudaError_t launch_ray_map(const BrickSummary* summ, const int32_t nb[3], bool plain_f, uint16_t* map,
                            cudaStream_t stream);
 // Reads the map of the volume as it is (launch_ray_map after its last change).
-// behind: the launch before this one on the stream is another ray cast of the
-// same volume, beside which this one may run.
+// link: FIRST and BEHIND casts of one volume, queued one after another on the
+// stream, run beside one another; the launch after the last of them finds all
+// of them done.
+enum class RayLink { ALONE, FIRST, BEHIND };
 cudaError_t launch_raycast(const RayConst& c, const float* F, const uint8_t* W, const uint32_t* C, const uint16_t* map,
-                           float* range, float* vertex, float* normal, uint32_t* rgbw, bool behind,
+                           float* range, float* vertex, float* normal, uint32_t* rgbw, RayLink link,
                            cudaStream_t stream);
 
 // ------------------------------------------------------- camera tracking --

@@ -25,7 +25,7 @@
 // through 512^3, 1064 -> 256 us and 5 us for the map; 1920x1080 through 192^3,
 // 1936 -> 689 us and 3 us; the three prediction levels of a tracked frame at
 // 512^3, 2454 -> 613 us one after another, about 430 us beside one another
-// (launch_raycast, behind).  Eight blocks per SM; 7, 10 and 12 were slower.
+// (launch_raycast, RayLink).  Eight blocks per SM; 7, 10 and 12 were slower.
 #include <cfloat>
 #include <cstdint>
 
@@ -227,22 +227,25 @@ __device__ __forceinline__ bool rc_pair(const RayConst& c, const float* __restri
     return true;
 }
 
+// CHAIN: the casts launched beside one another (launch_raycast, RayLink).
+// They read nothing of one another: the next one's blocks may start at once,
+// filling the SMs this one's last rays leave, and one block ends only after
+// the cast before it has, so the last cast's end is the end of all.  A cast
+// by itself runs without these, which held eight bytes more per thread
+// (spilled): 640x480 through 512^3 328 -> 310 us, 1920x1080 through 192^3
+// 883 -> 789 us; three chained casts 25 us less with one waiting thread
+// instead of all.
+template <bool CHAIN>
 __global__ void __launch_bounds__(RC_THREADS, 8) k_raycast(RayConst c, const float* __restrict__ F,
                                                         const uint8_t* __restrict__ W, const uint32_t* __restrict__ C,
                                                         const uint16_t* __restrict__ map, float* __restrict__ range,
                                                         float* __restrict__ vertex, float* __restrict__ normal,
                                                         uint32_t* __restrict__ rgbw) {
-    // Casts launched as a chain (launch_raycast, behind) read nothing of one
-    // another: the next one's blocks may start at once, filling the SMs this
-    // one's last rays leave; each ends after the one before it.
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if constexpr (CHAIN) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int x = blockIdx.x * RC_BX + (warp & 1) * 8 + (lane & 7);
     const int y = blockIdx.y * RC_BY + (warp >> 1) * 4 + (lane >> 3);
-    if (x >= c.width || y >= c.height) {
-        asm volatile("griddepcontrol.wait;" ::: "memory");
-        return;
-    }
+    if (x >= c.width || y >= c.height) return;
     const float fx = (float)x, fy = (float)y;
     const float dc0 = fmaf(c.Kinv[0], fx, fmaf(c.Kinv[1], fy, c.Kinv[2]));
     const float dc1 = fmaf(c.Kinv[3], fx, fmaf(c.Kinv[4], fy, c.Kinv[5]));
@@ -420,7 +423,9 @@ __global__ void __launch_bounds__(RC_THREADS, 8) k_raycast(RayConst c, const flo
         normal[3 * i + 2] = n[2];
     }
     if (rgbw) rgbw[i] = col;
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if constexpr (CHAIN) {
+        if (x == 0 && y == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+    }
 }
 
 }  // namespace
@@ -434,7 +439,7 @@ cudaError_t launch_ray_map(const BrickSummary* summ, const int32_t nb[3], bool p
 }
 
 cudaError_t launch_raycast(const RayConst& c, const float* F, const uint8_t* W, const uint32_t* C, const uint16_t* map,
-                           float* range, float* vertex, float* normal, uint32_t* rgbw, bool behind,
+                           float* range, float* vertex, float* normal, uint32_t* rgbw, RayLink link,
                            cudaStream_t stream) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((c.width + RC_BX - 1) / RC_BX, (c.height + RC_BY - 1) / RC_BY);
@@ -444,8 +449,9 @@ cudaError_t launch_raycast(const RayConst& c, const float* F, const uint8_t* W, 
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = behind ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, k_raycast, c, F, W, C, map, range, vertex, normal, rgbw);
+    cfg.numAttrs = link == RayLink::BEHIND ? 1 : 0;
+    auto k = link == RayLink::ALONE ? k_raycast<false> : k_raycast<true>;
+    return cudaLaunchKernelEx(&cfg, k, c, F, W, C, map, range, vertex, normal, rgbw);
 }
 
 }  // namespace tsdf

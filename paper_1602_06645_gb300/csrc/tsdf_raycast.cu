@@ -95,8 +95,8 @@ extern "C" tsdf_status tsdf_raycast(tsdf_volume* v, const float K[9], const floa
         cudaError_t e = tsdf::launch_ray_map(v->vol.summ, v->nb, v->plain_f, v->scr.ray_map, v->stream);
         if (e == cudaSuccess)
             e = tsdf::launch_raycast(c, v->vol.F, v->vol.W, v->vol.C, v->scr.ray_map, (float*)o_range.dev,
-                                     (float*)o_vertex.dev, (float*)o_normal.dev, (uint32_t*)o_rgbw.dev, false,
-                                     v->stream);
+                                     (float*)o_vertex.dev, (float*)o_normal.dev, (uint32_t*)o_rgbw.dev,
+                                     tsdf::RayLink::ALONE, v->stream);
         for (Out* o : {&o_range, &o_vertex, &o_normal, &o_rgbw}) {
             if (e != cudaSuccess || !o->staged) continue;
             e = cudaMemcpyAsync(o->user, o->dev, o->bytes, cudaMemcpyDeviceToHost, v->stream);

@@ -160,7 +160,7 @@ extern "C" tsdf_status tsdf_track(tsdf_volume* v, const uint16_t* depth_mm, tsdf
     e = tsdf::launch_ray_map(v->vol.summ, v->nb, v->plain_f, v->scr.ray_map, v->stream);
     for (int l = 0; l < p.levels && e == cudaSuccess; ++l)
         e = tsdf::launch_raycast(rc[l], v->vol.F, v->vol.W, v->vol.C, v->scr.ray_map, nullptr, PVl[l], PNl[l], nullptr,
-                                 l > 0, v->stream);
+                                 l > 0 ? tsdf::RayLink::BEHIND : tsdf::RayLink::FIRST, v->stream);
     if (e != cudaSuccess) return cuda_fail(v, e, "track: prediction");
     int step = 0;
     int step_level[TSDF_TRACK_MAX_STEPS];
