@@ -384,7 +384,10 @@ def run_ours(args):
     peaks, peak_kind = measured_peaks()
     hbm = float(peaks.get("hbm_gbs", 6800.0))
     K = max(args.steps, 1)
-    geo_bytes = 10.0 * st.total_geo_updated / K            # F (4 B) + w (1 B), read and written
+    # w (1 B) of every updated voxel, read and written, and with culling off its F (4 B) too.  With culling on,
+    # bricks in front of every measurement (most of them) need no F; the counters do not tell the others'
+    # voxels apart, so their F is left out: a lower bound.
+    geo_bytes = (10.0 if args.dense else 2.0) * st.total_geo_updated / K
     band_bytes = 5.0 * 729 * st.total_col_bricks / K        # geometry tile (9^3 F + w) per candidate brick
     vox_bytes = 8.0 * st.total_col_updated / K              # packed RGBW, read and written
     kern_bytes = {"geometry": geo_bytes, "colour_band": band_bytes, "colour_voxels": vox_bytes}
@@ -605,10 +608,11 @@ def run_batched(args):
     # the job's units over all ranks
     _, (nominal_all, geo_upd, col_upd, col_bricks) = reduce_over_ranks(dist, "cuda", [],
                                                                        [nominal, geo_upd, col_upd, col_bricks])
-    # algorithmic bytes of the step: F and w read and written per updated
-    # geometry voxel, the 9^3 geometry tile (F and w) per colour-candidate
-    # brick, the packed colour read and written per updated colour voxel
-    step_bytes = 10.0 * geo_upd + 5.0 * 729 * col_bricks + 8.0 * col_upd
+    # algorithmic bytes of the step: w read and written per updated geometry
+    # voxel (F of open bricks is neither: a lower bound), the 9^3 geometry tile
+    # (F and w) per colour-candidate brick, the packed colour read and written
+    # per updated colour voxel
+    step_bytes = 2.0 * geo_upd + 5.0 * 729 * col_bricks + 8.0 * col_upd
     peaks, peak_kind = measured_peaks()
     hbm = float(peaks["hbm_gbs"])
     # per GPU: the job's bytes over the GPUs
@@ -774,7 +778,7 @@ def run_raycast(args):
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "config": {"workload": seq.name + "_raycast_640x480", "fused_frames": n_fuse, "near_far_m": [0.1, 4.0],
                    "l2": "flushed between steps (256 MiB write)"},
-        "hit_fraction": float(torch.stack(hits).float().mean()), "gpu_launches": K, "clocks": ck.result,
+        "hit_fraction": float(torch.stack(hits).float().mean()), "gpu_launches": 2 * K, "clocks": ck.result,
     }
     vol.close()
     print(json.dumps(line), flush=True)
@@ -835,7 +839,7 @@ def run_mesh(args):
         "config": {"workload": seq.name + "_mesh_texture", "fused_frames": n_fuse, "size_pixel_m": size,
                    "l2": "flushed between steps (256 MiB write)"},
         "triangles": n_tri, "texels": n_tex, "mesh_ms": sum(mesh_ms) / K, "texture_ms": sum(tex_ms) / K,
-        "texels_per_s": n_tex * K / (sum(tex_ms) / 1e3), "gpu_launches": 7 * K, "clocks": ck.result,
+        "texels_per_s": n_tex * K / (sum(tex_ms) / 1e3), "gpu_launches": 6 * K, "clocks": ck.result,
     }
     vol.close()
     print(json.dumps(line), flush=True)
@@ -895,7 +899,7 @@ def run_track(args):
                    "l2": "not flushed: each call rebuilds its pyramid, maps and predictions"},
         "pose_error_mm": {"median": float(np.median(e[:, 0])), "max": float(e[:, 0].max())},
         "pose_error_deg": {"median": float(np.median(e[:, 1])), "max": float(e[:, 1].max())},
-        "correspondences_last_step": int(np.median(corr)), "gpu_launches": (3 * 2 + 3 + 19 * 2) * K,
+        "correspondences_last_step": int(np.median(corr)), "gpu_launches": (3 + 3 + 1 + 3 + 19) * K,
         "clocks": ck.result,
     }
     vol.close()

@@ -4,7 +4,8 @@
 // Order per frame on one stream:
 //   k_depth_tiles   min / max valid depth of each 8x8 depth tile; zeroes counters
 //   k_bricks        conservative per-brick visibility -> geometry and visible lists
-//   k_geometry      persistent: TSDF update of each listed brick, brick summaries
+//   k_geometry      persistent: TSDF update of each listed brick, brick summaries; bricks in
+//                   front of every measurement ("open") need only their weights
 //   k_colour_list   visible bricks whose owned cells (the brick and the first layers
 //                   of its + neighbours) can hold |F| <= band
 //   k_colour_band   one warp per listed brick: stages its geometry tile, finds
@@ -24,7 +25,7 @@
 namespace tsdf {
 namespace {
 
-constexpr int GEO_THREADS = 128;  // 4 voxels per thread, one brick per block iteration
+constexpr int GEO_THREADS = 128;  // 4 warps, one brick per warp
 constexpr int COL_THREADS = 128;  // 4 warps, one colour work item per warp
 constexpr int TILE_G = BRICK + 1;          // geometry tile edge: the brick + the next bricks' first voxel layer
 constexpr int TILE_G3 = TILE_G * TILE_G * TILE_G;
@@ -34,9 +35,8 @@ constexpr int CELLS3 = CELLS * CELLS * CELLS;
 // ------------------------------------------------------- depth tiles ----
 // Per 8x8-pixel tile the min / max valid depth (mm); with depth_m, also the
 // depth in metres per pixel as the geometry update reads it: RN(D * 0.001),
-// -inf where D = 0.  One warp per strip of four tiles (32 x 8 pixels): lane
-// x reads column x of the strip row by row (64 contiguous bytes per row),
-// and lanes 8t .. 8t + 7 reduce tile t.  Blocks are two warps: the next
+// -inf where D = 0.  One warp per strip of four tiles (32 x 8 pixels).
+// Blocks are two warps: the next
 // frame's tiles run beside the current frame's colour kernels, whose blocks
 // leave only a few thousand registers of an SM free.
 constexpr int TILES_THREADS = 64;
