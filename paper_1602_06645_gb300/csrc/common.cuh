@@ -42,6 +42,8 @@ struct FrameConst {
     int32_t record_mode;   // 1: the band kernel only records (adjoint gate recording); no colour update
     int32_t zoff_g, zoff_c;  // z-slab: global z index of held geometry / colour z = 0 (whole volume: 0)
     uint32_t pix_bias;       // 0x4B000000 (dw + 1) mod 2^32: pixel index from the bits of u + 2^23, v + 2^23
+    uint32_t max_weight4;    // max_weight in each of four bytes, and its low seven bits (see weights_after)
+    uint32_t max_weight4_low;
     uint32_t frame_tag;      // nonzero, different in consecutive frames: marks this frame's ready-queue entries
     int32_t open_bricks;     // 1: open bricks (see brick_flags) take their own geometry update
     int32_t fused;           // 1: the frame runs as one fused launch (k_fused) instead of the kernel chain

@@ -637,6 +637,22 @@ __device__ __forceinline__ uint32_t zero_bytes(uint32_t v) {
     return ~(((v & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | v | 0x7F7F7F7Fu) >> 7;
 }
 
+// Four weights (bytes of w) after an update of the voxels in upm (bit i: byte
+// i): min(w + 1, max_weight) there, the others as they are.  A weight may lie
+// above the limit (a restored volume, a caller's array, a limit lowered between
+// calls).  Byte by byte without a carry: ge says w >= limit, from the low seven
+// bits of both ((w | 0x80) - limit cannot borrow) and their top bits; below the
+// limit 1 is added, from it on the limit is taken.  The limit's words come with
+// the frame: formed here they cost k_geometry registers it does not have (76
+// bytes spilled per thread instead of none).
+__device__ __forceinline__ uint32_t weights_after(const FrameConst& c, uint32_t w, uint32_t upm) {
+    const uint32_t upb = (upm * 0x00204081u) & 0x01010101u;  // bit i of upm -> byte i
+    const uint32_t h = (w | 0x80808080u) - c.max_weight4_low;
+    const uint32_t ge = (((h & w) | ((h | w) & ~c.max_weight4)) >> 7) & upb;  // updated bytes at or above the limit
+    const uint32_t to_limit = ge * 0xFFu;
+    return ((w + (upb ^ ge)) & ~to_limit) | (c.max_weight4 & to_limit);
+}
+
 // Minimum / maximum of a float over the warp (sm_100 warp reduction; no NaN
 // reaches it here).
 __device__ __forceinline__ float warp_min(float v) {
@@ -688,7 +704,7 @@ __device__ __forceinline__ void geometry_update(const FrameConst& c, float* Fb, 
     const float2 pxp[2] = {make_float2(fmaf(gxf + 0.5f, c.s_g, c.origin[0]), fmaf(gxf + 1.5f, c.s_g, c.origin[0])),
                            make_float2(fmaf(gxf + 2.5f, c.s_g, c.origin[0]), fmaf(gxf + 3.5f, c.s_g, c.origin[0]))};
     const float gzf = (float)(at.bz * BRICK + lz + c.zoff_g) + 0.5f;  // centre at the global index
-    const uint32_t maxw = (uint32_t)c.max_weight, maxw4 = maxw * 0x01010101u;
+    const uint32_t maxw = (uint32_t)c.max_weight, maxw4 = c.max_weight4;
     // min / max of F over this lane's observed voxels: all of them, and those
     // on the brick faces (band flags): this lane's x face is its voxel i = 0
     // (lx = 0, the -x face) or i = 3 (lx = 4, +x), its z face its group j = 0
@@ -794,9 +810,7 @@ __device__ __forceinline__ void geometry_update(const FrameConst& c, float* Fb, 
                     fo[i] = (up || wb[k] != 0x4B000000u) && valid[k] ? fv[i] : qnan;  // observed after the update
                 }
             }
-            // w <- min(w + 1, max_weight): +1 in the updated bytes that are below the cap
-            const uint32_t upb = (upm * 0x00204081u) & 0x01010101u;  // bit i of upm -> byte i
-            const uint32_t wn = w_old + (upb & ~zero_bytes(w_old ^ maxw4));
+            const uint32_t wn = weights_after(c, w_old, upm);
             // in-volume voxels only: a byte outside the volume reads as observed and at the cap
             const uint32_t wq = ALIGNED ? wn : (wn & inside) | (maxw4 & ~inside);
             unobserved = unobserved || any_zero_byte(wq);
@@ -952,15 +966,13 @@ __device__ __forceinline__ void geometry_open(const FrameConst& c, const Volumes
     count += __popc(upd);
     if (!__any_sync(0xffffffffu, upd != 0u)) return;  // nothing changed: the summary stays
     ++changed;
-    const uint32_t maxw = (uint32_t)c.max_weight, maxw4 = maxw * 0x01010101u;
-    // w <- min(w + 1, max_weight) of the updated voxels, as in geometry_update
+    const uint32_t maxw = (uint32_t)c.max_weight, maxw4 = c.max_weight4;
     uint32_t wn[4], below = 0;
     bool hole = false;  // an unobserved voxel before the update
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         const uint32_t upm = (upd >> (4 * j)) & 15u, w_old = wv[j];
-        const uint32_t upb = (upm * 0x00204081u) & 0x01010101u;  // bit i of upm -> byte i
-        wn[j] = w_old + (upb & ~zero_bytes(w_old ^ maxw4));
+        wn[j] = weights_after(c, w_old, upm);
         hole = hole || any_zero_byte(w_old);
         below |= wn[j] ^ maxw4;
         if (upm) *reinterpret_cast<uint32_t*>(Wb + 128 * j) = wn[j];

@@ -169,6 +169,8 @@ void frame_constants(const tsdf_volume* v, const float Kd[9], const float Kr[9],
     c.kr_pinhole = pinhole(Kr);
     c.kdi_pinhole = c.Kdi[1] == 0.0f && c.Kdi[3] == 0.0f && c.Kdi[6] == 0.0f && c.Kdi[7] == 0.0f && c.Kdi[8] == 1.0f;
     c.max_weight = v->max_weight;
+    c.max_weight4 = (uint32_t)v->max_weight * 0x01010101u;
+    c.max_weight4_low = c.max_weight4 & 0x7F7F7F7Fu;
     c.free_space = v->free_space;
     c.sample_mode = v->sample_mode;
     c.colour_mode = v->colour_mode;
