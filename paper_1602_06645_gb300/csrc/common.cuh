@@ -51,6 +51,8 @@ struct FrameConst {
 
 // Min/max of F over observed voxels (w > 0) and min of w over the in-volume
 // voxels of one geometry brick.  No observed voxel: fmin = +inf, fmax = -inf.
+// wmin = 0 where some voxel may be unobserved, max_weight only where every w is
+// (it tells no more: other values need not be the minimum).
 // flags: bit 0 / 1 = some observed voxel has F <= band + eps / F >= -band - eps;
 // bits 2 + 2f / 3 + 2f = the same over face layer f (-x, +x, -y, +y, -z, +z).
 struct BrickSummary {
@@ -215,7 +217,7 @@ cudaError_t launch_from_linear_u32(uint32_t* brick, const uint32_t* lin, const i
                                    cudaStream_t stream);
 // Sets *odd_f (zeroed first) to 1 if some voxel's F is no number within PLAIN_F.
 cudaError_t launch_recompute_summaries(const float* F, const uint8_t* W, BrickSummary* summ, const int32_t ng[3],
-                                       float band, uint32_t* odd_f, cudaStream_t stream);
+                                       float band, int32_t max_weight, uint32_t* odd_f, cudaStream_t stream);
 constexpr float PLAIN_F = 1e30f;
 constexpr float CELL_EPS = 1e-5f;  // bound on trilinear overshoot of the corner range
 

@@ -85,18 +85,19 @@ cudaError_t convert(T* brick, T* lin, const int32_t dims[3], int z0, int z1, cud
 }
 
 // Brick summaries: min/max of F over observed voxels, min of w over in-volume
-// voxels and the band flags (what the geometry kernel maintains).  Bound by
-// HBM (5 B per voxel).  One warp per brick with the geometry kernel's lane
-// layout (lane l: voxels 4 (l + 32 j) .. + 3, j = 0..3), all eight 16- and
-// 4-byte reads of a lane issued together; the flags come from the minima and
-// maxima over the lane's faces: 118 us at 512^3 (5.7 TB/s); one block per
-// brick with scalar reads and a shared-memory reduction took 235 us.
+// voxels (never max_weight where some w lies above it) and the band flags
+// (what the geometry kernel maintains).  Bound by HBM (5 B per voxel).  One
+// warp per brick with the geometry kernel's lane layout (lane l: voxels
+// 4 (l + 32 j) .. + 3, j = 0..3), all eight 16- and 4-byte reads of a lane
+// issued together; the flags come from the minima and maxima over the lane's
+// faces: 118 us at 512^3 (5.7 TB/s); one block per brick with scalar reads and
+// a shared-memory reduction took 235 us.
 constexpr int SUM_WARPS = 8;
 __global__ void __launch_bounds__(SUM_WARPS * 32) k_summaries(const float* __restrict__ F,
                                                               const uint8_t* __restrict__ W,
                                                               BrickSummary* __restrict__ summ, int nx, int ny, int nz,
                                                               int nbx, int nby, uint32_t nbt, float band,
-                                                              uint32_t* __restrict__ odd_f) {
+                                                              uint32_t max_weight, uint32_t* __restrict__ odd_f) {
     const uint32_t b = blockIdx.x * SUM_WARPS + (threadIdx.x >> 5);
     if (b >= nbt) return;
     const int lane = threadIdx.x & 31;
@@ -112,7 +113,7 @@ __global__ void __launch_bounds__(SUM_WARPS * 32) k_summaries(const float* __res
     }
     const float inf = __int_as_float(0x7f800000), qnan = __int_as_float(0x7fffffff);
     float mn = inf, mx = -inf, mn_xf = inf, mx_xf = -inf, mn_zf = inf, mx_zf = -inf;
-    uint32_t wmn = 0xFFFFFFFFu;
+    uint32_t wmn = 0xFFFFFFFFu, wmx = 0u;
     bool odd = false;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -124,6 +125,7 @@ __global__ void __launch_bounds__(SUM_WARPS * 32) k_summaries(const float* __res
             const bool vox = in && bx * BRICK + lx + i < nx;
             const uint32_t wi = (w[j] >> (8 * i)) & 0xFFu;
             wmn = min(wmn, vox ? wi : 0xFFFFFFFFu);
+            wmx = max(wmx, vox ? wi : 0u);
             odd = odd || (vox && !(fabsf(fv[i]) <= PLAIN_F));
             const float v = vox && wi ? fv[i] : qnan;  // fminf / fmaxf pass over a NaN
             gmn = fminf(gmn, v);
@@ -148,6 +150,9 @@ __global__ void __launch_bounds__(SUM_WARPS * 32) k_summaries(const float* __res
     if (__any_sync(0xffffffffu, odd) && lane == 0) *odd_f = 1u;
     flags = __reduce_or_sync(0xffffffffu, flags);
     wmn = __reduce_min_sync(0xffffffffu, wmn);
+    // a weight above the limit comes down to it at its next update: the brick
+    // is not saturated, which wmin == max_weight would say
+    if (__reduce_max_sync(0xffffffffu, wmx) > max_weight && wmn == max_weight) ++wmn;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
@@ -186,14 +191,14 @@ cudaError_t launch_from_linear_u32(uint32_t* b, const uint32_t* l, const int32_t
 }
 
 cudaError_t launch_recompute_summaries(const float* F, const uint8_t* W, BrickSummary* summ, const int32_t ng[3],
-                                       float band, uint32_t* odd_f, cudaStream_t stream) {
+                                       float band, int32_t max_weight, uint32_t* odd_f, cudaStream_t stream) {
     const cudaError_t e = cudaMemsetAsync(odd_f, 0, sizeof(uint32_t), stream);
     if (e != cudaSuccess) return e;
     const int nbx = (ng[0] + BRICK - 1) / BRICK, nby = (ng[1] + BRICK - 1) / BRICK, nbz = (ng[2] + BRICK - 1) / BRICK;
     const int64_t nbt = (int64_t)nbx * nby * nbz;
     if (nbt > 0)
         k_summaries<<<(unsigned)((nbt + SUM_WARPS - 1) / SUM_WARPS), SUM_WARPS * 32, 0, stream>>>(
-            F, W, summ, ng[0], ng[1], ng[2], nbx, nby, (uint32_t)nbt, band, odd_f);
+            F, W, summ, ng[0], ng[1], ng[2], nbx, nby, (uint32_t)nbt, band, (uint32_t)max_weight, odd_f);
     return cudaGetLastError();
 }
 

@@ -91,3 +91,30 @@ def test_handle_weights_above_the_limit(dims, mode, max_weight):
             F, W, _ = v.read()
         np.testing.assert_array_equal(W, o.W, err_msg=str(form))
         np.testing.assert_array_equal(F, o.F, err_msg=str(form))
+
+
+@pytest.mark.parametrize("above", [0, 3, 191])
+@pytest.mark.parametrize("dims", [(32, 32, 32), (30, 21, 43)])
+def test_free_space_above_the_limit_is_not_saturated(dims, above):
+    """Free space (F = 1) whose smallest weight is the limit: it is left out of
+    the update only where no weight lies above the limit."""
+    s, limit = float(np.float32(0.6 / max(dims))), 64
+    shape = dims[::-1]
+    F0, W0 = np.ones(shape, np.float32), np.full(shape, limit, np.uint8)
+    W0[::5, ::3, ::5] += above
+    rgb = np.zeros((120, 160, 3), np.uint8)
+    o = oracle.Oracle(dims, dims, s, 3 * s, limit, n_threads=4)
+    o.F[...], o.W[...] = F0, W0
+    for k in range(2):
+        o.integrate(depth(2500, k), rgb, K, KR, POSES[k], TDR)
+    assert above == 0 or ((o.W == limit) & (W0 > limit)).sum() > 100
+    for form in (dict(culling=True), dict(culling=False), dict(schedule=T.TSDF_SCHEDULE_FUSED)):
+        with T.Volume(dims, dims, s, 3 * s, limit, **form) as v:
+            v.write(F0, W0)
+            for k in range(2):
+                v.integrate(depth(2500, k), rgb, K, KR, POSES[k], TDR)
+            F, W, _ = v.read()
+            if form.get("culling") and above == 0:
+                assert v.stats().geo_bricks == 0  # saturated free space
+        np.testing.assert_array_equal(W, o.W, err_msg=str(form))
+        np.testing.assert_array_equal(F, o.F, err_msg=str(form))
