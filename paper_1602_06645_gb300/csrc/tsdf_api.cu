@@ -828,9 +828,12 @@ tsdf_status tsdf_write(tsdf_volume* v, const float* tsdf, const uint8_t* w_geo, 
     tsdf_status s = write_volume<float>(v, v->vol.F, tsdf, v->ng, launch_from_linear_f32);
     if (s == TSDF_OK) s = write_volume<uint8_t>(v, v->vol.W, w_geo, v->ng, launch_from_linear_u8);
     if (s == TSDF_OK) s = write_volume<uint32_t>(v, v->vol.C, rgbw, v->nc, launch_from_linear_u32);
-    if (s != TSDF_OK) return s;
+    // A restore that failed half way has changed some of the values all the
+    // same: the summaries and err[1] are made for what the volumes now hold.
     cudaError_t e = launch_recompute_summaries(v->vol.F, v->vol.W, v->vol.summ, v->ng, v->band, v->max_weight,
                                                v->scr.err + 1, v->stream);
+    if (e != cudaSuccess) cudaMemsetAsync(v->scr.err + 1, 1, sizeof(uint32_t), v->stream);  // nothing is known of F
+    if (s != TSDF_OK) return s;
     if (e != cudaSuccess) return cuda_fail(v, e, "summaries");
     return check_device_error(v);
 }
