@@ -45,6 +45,7 @@ struct FrameConst {
     uint32_t max_weight4;    // max_weight in each of four bytes, and its low seven bits (see weights_after)
     uint32_t max_weight4_low;
     uint32_t frame_tag;      // nonzero, different in consecutive frames: marks this frame's ready-queue entries
+    int32_t footprint_holds; // 1: no voxel leaves its brick's footprint by rounding (footprint_bound.h)
     int32_t open_bricks;     // 1: open bricks (see brick_flags) take their own geometry update
     int32_t fused;           // 1: the frame runs as one fused launch (k_fused) instead of the kernel chain
 };

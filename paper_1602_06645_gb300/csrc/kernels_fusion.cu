@@ -260,7 +260,8 @@ __device__ __forceinline__ void depth_flags(const FrameConst& c, const BrickSumm
         if (sat && ahead) f.geo = false;
         // every measurement under an open brick puts its voxels at t = 1,
         // and every voxel observed so far is at F = 1 (or none is): the
-        // update only counts (see geometry_open)
+        // update only counts (see geometry_open).  open_bricks implies that
+        // the footprint holds, so zmax bounds every voxel's computed depth
         f.open = c.open_bricks && ahead && (ones || !(s.fmin <= FLT_MAX));
         // colour: Eq. 7 needs |Z - d| <= sigma (pinhole K_c: the back-projected
         // point has Z = d), so a brick wholly nearer than the nearest depth
@@ -279,9 +280,10 @@ __device__ __forceinline__ PixelBox pixel_box(const FrameConst& c, const Footpri
     if (!f.straddle) {
         // every corner is in front of the camera and the footprint lies
         // more than a pixel inside the image: every voxel of the brick is
-        // in front and projects into the image (the geometry update then
-        // skips its per-voxel image tests)
-        inner = f.umin > 1.0f && f.vmin > 1.0f && f.umax < (float)c.dw - 2.0f && f.vmax < (float)c.dh - 2.0f;
+        // in front and projects into the image, rounding included (the
+        // geometry update then skips its per-voxel image tests)
+        inner = c.footprint_holds && f.umin > 1.0f && f.vmin > 1.0f && f.umax < (float)c.dw - 2.0f &&
+                f.vmax < (float)c.dh - 2.0f;
         // clamp before converting so the integer bounds cannot overflow
         const float umin = fmaxf(f.umin, -4.0f), umax = fminf(f.umax, (float)c.dw + 4.0f);
         const float vmin = fmaxf(f.vmin, -4.0f), vmax = fminf(f.vmax, (float)c.dh + 4.0f);
@@ -2605,7 +2607,9 @@ cudaError_t launch_geometry_static(const FrameConst& c, float* F, uint8_t* W, co
         e = launch_chained(small ? k_bricks_static<true> : k_bricks_static<false>,
                            dim3(((small ? nbt * 8u : nbt) + 255) / 256), dim3(256), 0, stream, c, tiles, ctr, geo_list);
     if (e != cudaSuccess) return e;
-    const bool rows = c.ng[0] % 4 == 0 && ((uintptr_t)F & 15u) == 0 && ((uintptr_t)W & 3u) == 0;
+    // Where rounding may move a voxel out of its brick's footprint (coordinates
+    // large against the voxel, or not finite), every voxel is tested by itself.
+    const bool rows = c.footprint_holds && c.ng[0] % 4 == 0 && ((uintptr_t)F & 15u) == 0 && ((uintptr_t)W & 3u) == 0;
     const bool aligned = rows && c.ng[0] % BRICK == 0 && c.ng[1] % BRICK == 0 && c.ng[2] % BRICK == 0;
     void (*k)(FrameConst, float*, uint8_t*, const uint16_t*, Counters*, const uint32_t*) =
         rows ? (aligned ? (c.kd_pinhole ? k_geometry_rows<true, true, true> : k_geometry_rows<false, true, true>)

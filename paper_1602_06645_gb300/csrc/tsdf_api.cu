@@ -18,6 +18,7 @@
 #include "../../include/tsdf.h"
 #include "api_internal.h"
 #include "common.cuh"
+#include "footprint_bound.h"
 
 using namespace tsdf;
 
@@ -178,16 +179,9 @@ void frame_constants(const tsdf_volume* v, const float Kd[9], const float Kr[9],
     // Beyond the farthest depth by more than max(mu, sigma) nothing can pass
     // the sdf >= -mu test nor (pinhole K_c: the back-projected point has
     // Z = d) the sigma gate; 2 mm covers binary32 rounding many times over.
-    // Open bricks rest on a margin of 2 mm between binary32 depths computed in
-    // two ways; each is off by less than 1e-6 of the coordinates that enter it.
-    float far_out = 0.0f;
-    for (int a = 0; a < 3; ++a) {
-        const float end = v->origin[a] + (float)(v->ng[a] + (a == 2 ? v->zoff_g : 0)) * v->s_g;
-        far_out = std::fmax(far_out, std::fmax(std::fabs(v->origin[a]), std::fabs(end)));
-        far_out = std::fmax(far_out, std::fabs(Twd[a * 4 + 3]));
-    }
-    // Their pixel indices are binary32 integers.
-    c.open_bricks = v->plain_f && v->free_space && far_out <= 500.0f && (int64_t)dw * dh < (1 << 23) ? 1 : 0;
+    c.footprint_holds = footprint_holds(c.R, c.t, c.Kd, c.Kdi, c.origin, c.nb, c.zoff_g, c.s_g) ? 1 : 0;
+    // The pixel indices of open bricks are binary32 integers.
+    c.open_bricks = v->plain_f && v->free_space && c.footprint_holds && (int64_t)dw * dh < (1 << 23) ? 1 : 0;
     c.cull_behind = c.kdi_pinhole ? std::fmax(v->mu, v->sigma) + 2e-3f : INFINITY;
 }
 
