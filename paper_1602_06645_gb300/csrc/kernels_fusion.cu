@@ -681,9 +681,9 @@ struct DepthM {
 
 // TSDF update of geometry brick `at` by one warp (lane = lane index) from its
 // F and w already loaded (f, wv: this lane's four groups, the j-th at Fb and Wb
-// + step j); writes the changed groups and, unless summ is null, the brick
-// summary.  Adds the number of updated voxels to count
-// and 1 to changed if any voxel changed.
+// + step j); writes the changed groups and the brick summary.  Adds the number
+// of updated voxels to count and 1 to changed if any voxel changed.  CALLERS:
+// the caller's volume, of which no summary is kept.
 //   D = depth at the nearest pixel of the voxel centre (Eq. 6); D = 0 skipped
 //   sdf = D * 0.001 - Z; sdf < -mu skipped; (free space off: sdf > mu skipped)
 //   t = min(1, sdf * (1/mu)); F <- fmaf(F, w, t) / (w + 1); w <- min(w+1, max_w)
@@ -691,7 +691,7 @@ struct DepthM {
 // (j = 0..3) of the brick: voxels 4q..4q+3, i.e. x in {0..3} or {4..7},
 // y = (l >> 1) & 7, z = (l >> 4) + 2 j.  Each group of the warp is 512
 // contiguous bytes of F and 128 of w.
-template <bool PINHOLE, bool FREE_SPACE, bool ALIGNED, bool INNER, typename Depth>
+template <bool PINHOLE, bool FREE_SPACE, bool ALIGNED, bool INNER, bool CALLERS, typename Depth>
 __device__ __forceinline__ void geometry_update(const FrameConst& c, float* Fb, uint8_t* Wb, int step,
                                                 BrickSummary* summ, Depth depth, const BrickAt& at, int lane,
                                                 const float4 (&f)[4], const uint32_t (&wv)[4], uint32_t& count,
@@ -800,7 +800,14 @@ __device__ __forceinline__ void geometry_update(const FrameConst& c, float* Fb, 
                 const float2 a = __ffma2_rn(make_float2(fin[2 * h], fin[2 * h + 1]), wf, t);
                 const float2 q = __fmul2_rn(a, y);
                 const float2 r = __ffma2_rn(nb, q, a);
-                const float2 fn = __ffma2_rn(r, y, q);
+                float2 fn = __ffma2_rn(r, y, q);
+                // A caller's F may be infinite or overflow in F w + t: the
+                // quotient is then that infinity, where the residual is not a
+                // number.
+                if (CALLERS) {
+                    fn.x = fabsf(a.x) <= FLT_MAX ? fn.x : a.x;
+                    fn.y = fabsf(a.y) <= FLT_MAX ? fn.y : a.y;
+                }
                 const float sd[2] = {sdf.x, sdf.y}, fnew[2] = {fn.x, fn.y};
                 const uint32_t wb[2] = {wb0, wb1};
 #pragma unroll
@@ -837,7 +844,7 @@ __device__ __forceinline__ void geometry_update(const FrameConst& c, float* Fb, 
         }
     }
     count += __popc(upd);
-    if (!summ) return;
+    if (CALLERS) return;
     // bricks where nothing changed keep their summary
     if (!__any_sync(0xffffffffu, upd != 0u)) return;
     ++changed;
@@ -881,8 +888,8 @@ __device__ __forceinline__ void geometry_brick(const FrameConst& c, const Volume
         f[j] = *reinterpret_cast<const float4*>(Fb + 128 * j);
         wv[j] = *reinterpret_cast<const uint32_t*>(Wb + 128 * j);
     }
-    geometry_update<PINHOLE, FREE_SPACE, ALIGNED, INNER>(c, Fb, Wb, 128, vol.summ, depth, at, lane, f, wv, count,
-                                                         changed);
+    geometry_update<PINHOLE, FREE_SPACE, ALIGNED, INNER, false>(c, Fb, Wb, 128, vol.summ, depth, at, lane, f, wv, count,
+                                                                changed);
 }
 
 // The depth at pixel 0x4B000000 + i of an image of less than 2^23 pixels, as a
@@ -2064,11 +2071,11 @@ __global__ void __launch_bounds__(GEO_THREADS, 4) k_geometry_rows(FrameConst c, 
             }
         }
         if (e & GEO_INNER)
-            geometry_update<PINHOLE, FREE_SPACE, ALIGNED, true>(c, F + o, W + o, step, nullptr, depth, at, lane, f, wv,
-                                                                count, changed);
+            geometry_update<PINHOLE, FREE_SPACE, ALIGNED, true, true>(c, F + o, W + o, step, nullptr, depth, at, lane,
+                                                                      f, wv, count, changed);
         else
-            geometry_update<PINHOLE, FREE_SPACE, ALIGNED, false>(c, F + o, W + o, step, nullptr, depth, at, lane, f, wv,
-                                                                 count, changed);
+            geometry_update<PINHOLE, FREE_SPACE, ALIGNED, false, true>(c, F + o, W + o, step, nullptr, depth, at, lane,
+                                                                       f, wv, count, changed);
     }
     count = __reduce_add_sync(0xffffffffu, count);
     if (lane == 0 && count) atomicAdd(&ctr->geo_updated, (unsigned long long)count);

@@ -1,5 +1,6 @@
 """The caller-owned geometry volume (tsdf_integrate_geometry_static) against
-the oracle far from the world's origin, and the handle's frames there."""
+the oracle where its kernels differ: values that overflow, a volume far from
+the world's origin (and the handle's frames there)."""
 import numpy as np
 import pytest
 
@@ -48,6 +49,19 @@ def check(dims, s, F0, W0, frames, Kd, poses, origin=None, max_weight=255):
 
 def zeros(dims):
     return np.zeros(dims[::-1], np.float32), np.zeros(dims[::-1], np.uint8)
+
+
+@pytest.mark.parametrize("dims", DIMS)
+def test_values_that_overflow(dims):
+    """F of infinite, huge and tiny magnitude and not a number: the average is
+    the IEEE fmaf(F, w, t) / (w + 1)."""
+    rng = np.random.default_rng(sum(dims))
+    odd = np.array([np.inf, -np.inf, np.nan, 3e38, -3e38, 1e-40, -1e-45, 2e-38], np.float32)
+    F0 = rng.uniform(-1, 1, dims[::-1]).astype(np.float32)
+    F0.reshape(-1)[::3] = rng.choice(odd, F0.reshape(-1)[::3].shape)
+    W0 = rng.integers(0, 256, dims[::-1]).astype(np.uint8)
+    s = float(np.float32(0.6 / max(dims)))
+    assert check(dims, s, F0, W0, [surface(k) for k in range(3)], K, POSES) > F0.size // 20
 
 
 def far_frames():
