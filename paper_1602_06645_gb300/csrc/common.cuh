@@ -197,7 +197,7 @@ cudaError_t launch_frame_post(const FrameConst& c, const Volumes& v, const Scrat
 cudaError_t launch_frame(const FrameConst& c, const Volumes& v, const Scratch& s, const uint16_t* depth,
                          const uint8_t* rgb, const LaunchGrids& g, cudaStream_t stream, cudaEvent_t* ev = nullptr);
 int geometry_blocks_per_sm();
-int geometry_linear_blocks_per_sm();  // the linear-volume kernels (the allocation-free entry point)
+int geometry_static_blocks_per_sm(bool rows);  // the allocation-free entry point: k_geometry_rows, k_geometry_linear
 int colour_blocks_per_sm();
 int voxel_blocks_per_sm();
 int fused_blocks_per_sm();
@@ -225,7 +225,8 @@ constexpr float CELL_EPS = 1e-5f;  // bound on trilinear overshoot of the corner
 // Geometry-only fusion of one frame into caller-owned linear x-fastest F / w
 // arrays, with caller-provided scratch (counters, depth tiles, brick list).
 cudaError_t launch_geometry_static(const FrameConst& c, float* F, uint8_t* W, const uint16_t* depth, Counters* ctr,
-                                   uint32_t* tiles, uint32_t* geo_list, int grid_geo, cudaStream_t stream);
+                                   uint32_t* tiles, uint32_t* geo_list, int grid_rows, int grid_linear,
+                                   cudaStream_t stream);
 // Frame constants of a volume description, by the same rules as tsdf_integrate.
 struct VolumeDesc {
     int32_t ng[3];

@@ -2085,7 +2085,11 @@ __global__ void __launch_bounds__(GEO_THREADS, 4) k_geometry_rows(FrameConst c, 
     if (lane == 0 && count) atomicAdd(&ctr->geo_updated, (unsigned long long)count);
 }
 
-// The same for any row length and alignment, a voxel at a time.
+// The same for any row length and alignment, a voxel at a time.  Bound by the
+// latency of its dependent reads, so its grid is the nine blocks per SM that
+// its own registers allow: one 640x480 frame into 319 x 320 x 320 voxels 196 us,
+// 509 x 512 x 512 694 us, against 256 and 918 with the four blocks per SM of
+// k_geometry_rows.
 template <bool PINHOLE>
 __global__ void __launch_bounds__(GEO_THREADS, 7) k_geometry_linear(FrameConst c, float* __restrict__ F,
                                                                  uint8_t* __restrict__ W,
@@ -2514,9 +2518,10 @@ int geometry_blocks_per_sm() {
     return n > 0 ? n : 1;
 }
 
-int geometry_linear_blocks_per_sm() {
+int geometry_static_blocks_per_sm(bool rows) {
     int n = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_geometry_rows<true, true, true>, GEO_THREADS, 0);
+    if (rows) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_geometry_rows<true, true, true>, GEO_THREADS, 0);
+    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_geometry_linear<true>, GEO_THREADS, 0);
     return n > 0 ? n : 1;
 }
 
@@ -2609,7 +2614,8 @@ cudaError_t launch_frame(const FrameConst& c, const Volumes& v, const Scratch& s
 }
 
 cudaError_t launch_geometry_static(const FrameConst& c, float* F, uint8_t* W, const uint16_t* depth, Counters* ctr,
-                                   uint32_t* tiles, uint32_t* geo_list, int grid_geo, cudaStream_t stream) {
+                                   uint32_t* tiles, uint32_t* geo_list, int grid_rows, int grid_linear,
+                                   cudaStream_t stream) {
     const uint32_t nbt = (uint32_t)c.nb[0] * c.nb[1] * c.nb[2];
     const bool small = nbt <= SMALL_BRICKS;
     cudaError_t e = launch_chained(k_depth_tiles, depth_tiles_grid(c), dim3(TILES_THREADS), 0, stream, c, depth, tiles,
@@ -2626,7 +2632,7 @@ cudaError_t launch_geometry_static(const FrameConst& c, float* F, uint8_t* W, co
         rows ? (aligned ? (c.kd_pinhole ? k_geometry_rows<true, true, true> : k_geometry_rows<false, true, true>)
                         : (c.kd_pinhole ? k_geometry_rows<true, true, false> : k_geometry_rows<false, true, false>))
              : (c.kd_pinhole ? k_geometry_linear<true> : k_geometry_linear<false>);
-    return launch_chained(k, dim3(grid_geo), dim3(GEO_THREADS), 0, stream, c, F, W, depth, ctr, geo_list);
+    return launch_chained(k, dim3(rows ? grid_rows : grid_linear), dim3(GEO_THREADS), 0, stream, c, F, W, depth, ctr, geo_list);
 }
 
 cudaError_t launch_frame_record(const FrameConst& c, const Volumes& v, const Scratch& s, const uint16_t* depth,

@@ -36,7 +36,7 @@ static __device__ __align__(256) unsigned char g_scratch[SCRATCH_BYTES];
 constexpr int MAX_DEVICES = 64;
 std::mutex g_mutex;
 void* g_scratch_dev[MAX_DEVICES];  // device address of g_scratch per device, set on first use
-int g_grid[MAX_DEVICES];
+int g_grid[MAX_DEVICES][2];  // persistent grids: single voxels, wide rows
 
 bool finite_n(const float* a, int n) {
     for (int i = 0; i < n; ++i)
@@ -90,7 +90,7 @@ extern "C" tsdf_status tsdf_integrate_geometry_static(const int32_t dims[3], flo
     }
 
     // once per device, with that device current: the device address of the
-    // scratch array and the persistent grid size.  The address belongs to the
+    // scratch array and the persistent grid sizes.  The address belongs to the
     // device's primary context: after cudaDeviceReset the cached value is
     // stale, so the library must not be used across a device reset.
     int dev = 0;
@@ -99,7 +99,7 @@ extern "C" tsdf_status tsdf_integrate_geometry_static(const int32_t dims[3], flo
         return TSDF_ERR_CUDA;
     }
     void* scratch = nullptr;
-    int grid = 0;
+    int grid[2] = {0, 0};
     {
         std::lock_guard<std::mutex> lock(g_mutex);
         if (!g_scratch_dev[dev]) {
@@ -113,11 +113,12 @@ extern "C" tsdf_status tsdf_integrate_geometry_static(const int32_t dims[3], flo
                 cudaGetLastError();
                 return TSDF_ERR_CUDA;
             }
-            g_grid[dev] = sms * geometry_linear_blocks_per_sm();
+            for (int rows = 0; rows < 2; ++rows) g_grid[dev][rows] = sms * geometry_static_blocks_per_sm(rows != 0);
             g_scratch_dev[dev] = p;
         }
         scratch = g_scratch_dev[dev];
-        grid = g_grid[dev];
+        grid[0] = g_grid[dev][0];
+        grid[1] = g_grid[dev][1];
     }
     unsigned char* base = static_cast<unsigned char*>(scratch);
     Counters* ctr = reinterpret_cast<Counters*>(base);  // zeroed by the first kernel of every call
@@ -134,7 +135,7 @@ extern "C" tsdf_status tsdf_integrate_geometry_static(const int32_t dims[3], flo
     desc.max_weight = max_weight;
     FrameConst c;
     geometry_frame_constants(desc, K_depth, T_world_depth, dsz.width, dsz.height, c);
-    cudaError_t e = launch_geometry_static(c, tsdf_dev, w_dev, depth_dev, ctr, tile_buf, list, grid,
+    cudaError_t e = launch_geometry_static(c, tsdf_dev, w_dev, depth_dev, ctr, tile_buf, list, grid[1], grid[0],
                                            (cudaStream_t)stream);
     if (e != cudaSuccess) return TSDF_ERR_CUDA;
     return TSDF_OK;
