@@ -1,6 +1,7 @@
 """The caller-owned geometry volume (tsdf_integrate_geometry_static) against
 the oracle where its kernels differ: values that overflow, a volume far from
-the world's origin (and the handle's frames there)."""
+the world's origin (and the handle's frames there), a depth camera that is no
+pinhole (and the handle's frames with one), stream capture."""
 import numpy as np
 import pytest
 
@@ -125,3 +126,78 @@ def test_coordinates_that_overflow(dims):
     pose = np.eye(4, dtype=np.float32)
     assert check(dims, 1e37, F0, W0, [inside_a_buffer(surface(0)).cpu().numpy().view(np.uint16)], K, [pose],
                  origin=[3e38, 3e38, 3e38]) == 0
+
+
+SKEWED = {"skew": [[60.0, 3.0, 39.0], [1.5, 55.0, 29.0], [0.0, 0.0, 1.0]],
+          "tilted": [[60.0, 0.5, 39.0], [0.2, 55.0, 29.0], [0.05, -0.03, 1.1]]}
+
+
+@pytest.mark.parametrize("form", sorted(SKEWED))
+@pytest.mark.parametrize("dims", DIMS)
+def test_depth_camera_that_is_no_pinhole(dims, form):
+    s = float(np.float32(0.6 / max(dims)))
+    Kd = np.array(SKEWED[form], np.float32)
+    F0, W0 = zeros(dims)
+    assert check(dims, s, F0, W0, [surface(k) for k in range(3)], Kd, POSES) > F0.size // 20
+
+
+def test_captured_calls():
+    """Two chained calls captured in a graph, replayed on other depths."""
+    dims, s = (64, 64, 64), float(np.float32(0.6 / 64))
+    org = [-0.5 * m * s for m in dims]
+    F, W = (torch.from_numpy(a).cuda() for a in zeros(dims))
+    d = [dev(surface(k)) for k in range(2)]
+    call = lambda k, st: T.tsdf_integrate_geometry_static(dims, s, 3 * s, 64, org, F, W, d[k], K, POSES[k], st)  # noqa: E731
+    call(0, torch.cuda.current_stream().cuda_stream)  # the scratch array's address is looked up before a capture
+    torch.cuda.synchronize()
+    F.zero_(), W.zero_()
+    g, st = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g, stream=st):
+        call(0, st.cuda_stream)
+        call(1, st.cuda_stream)
+    o = oracle.Oracle(dims, dims, s, 3 * s, 64, n_threads=4)
+    for r in range(3):
+        for k in range(2):
+            m = surface(10 * r + k)
+            d[k].copy_(dev(m))
+            o.integrate_geometry(m, K, POSES[k])
+        torch.cuda.synchronize()
+        g.replay()
+        torch.cuda.synchronize()
+        np.testing.assert_array_equal(W.cpu().numpy(), o.W)
+        np.testing.assert_array_equal(F.cpu().numpy(), o.F)
+
+
+@pytest.mark.parametrize("form", sorted(SKEWED))
+@pytest.mark.parametrize("dims", [(32, 32, 32), (30, 21, 43)])
+@pytest.mark.parametrize("mm", [0, 2500])
+def test_handle_with_a_depth_camera_that_is_no_pinhole(dims, form, mm):
+    """mm 2500: a wall behind the volume, so its bricks lie in front of every measurement."""
+    s = float(np.float32(0.6 / max(dims)))
+    Kd = np.array(SKEWED[form], np.float32)
+    Kr, Tdr = synth.intrinsics(120.0, 110.0, 79.0, 59.0), synth.rig_depth_to_rgb()
+    rgb = np.random.default_rng(5).integers(0, 256, (120, 160, 3)).astype(np.uint8)
+    frames = []
+    for k in range(6):
+        d = surface(k)
+        frames.append(np.where(d > 0, mm, 0).astype(np.uint16) if mm else d)
+    o = oracle.Oracle(dims, dims, s, 3 * s, 4, n_threads=4)
+    for k, d in enumerate(frames):
+        o.integrate(d, rgb, Kd, Kr, POSES[k % 3], Tdr)
+    assert (o.W > 0).mean() > 0.2
+    for form in ("chain", "dense", "batch"):
+        with T.Volume(dims, dims, s, 3 * s, 4, culling=form != "dense") as v:
+            b = T.Batch([v]) if form == "batch" else None
+            for k, d in enumerate(frames):
+                if b:
+                    b.integrate([(dev(d), torch.from_numpy(rgb).cuda(), Kd, Kr, POSES[k % 3], Tdr)])
+                    b.synchronize()
+                else:
+                    v.integrate(d, rgb, Kd, Kr, POSES[k % 3], Tdr)
+            got = v.read()
+            if b:
+                b.close()
+        np.testing.assert_array_equal(got[1], o.W, err_msg=form)
+        np.testing.assert_array_equal(got[0], o.F, err_msg=form)
+        np.testing.assert_array_equal(got[2], o.C, err_msg=form)
