@@ -2043,7 +2043,7 @@ __global__ void __launch_bounds__(256) k_bricks_static(FrameConst c, const uint3
 // 4-byte (w) boundaries: a lane's four voxels are then one access, and two
 // voxels go through each instruction (128^3, one 640x480 frame: 25 -> 7.7 us;
 // four blocks per SM, the registers of both, without spills).
-template <bool PINHOLE, bool FREE_SPACE, bool ALIGNED>
+template <bool PINHOLE, bool ALIGNED>
 __global__ void __launch_bounds__(GEO_THREADS, 4) k_geometry_rows(FrameConst c, float* __restrict__ F,
                                                                  uint8_t* __restrict__ W,
                                                                  const uint16_t* __restrict__ depth_mm,
@@ -2075,11 +2075,11 @@ __global__ void __launch_bounds__(GEO_THREADS, 4) k_geometry_rows(FrameConst c, 
             }
         }
         if (e & GEO_INNER)
-            geometry_update<PINHOLE, FREE_SPACE, ALIGNED, true, true>(c, F + o, W + o, step, nullptr, depth, at, lane,
-                                                                      f, wv, count, changed);
+            geometry_update<PINHOLE, true, ALIGNED, true, true>(c, F + o, W + o, step, nullptr, depth, at, lane, f, wv,
+                                                                count, changed);
         else
-            geometry_update<PINHOLE, FREE_SPACE, ALIGNED, false, true>(c, F + o, W + o, step, nullptr, depth, at, lane,
-                                                                       f, wv, count, changed);
+            geometry_update<PINHOLE, true, ALIGNED, false, true>(c, F + o, W + o, step, nullptr, depth, at, lane, f, wv,
+                                                                 count, changed);
     }
     count = __reduce_add_sync(0xffffffffu, count);
     if (lane == 0 && count) atomicAdd(&ctr->geo_updated, (unsigned long long)count);
@@ -2520,7 +2520,7 @@ int geometry_blocks_per_sm() {
 
 int geometry_static_blocks_per_sm(bool rows) {
     int n = 0;
-    if (rows) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_geometry_rows<true, true, true>, GEO_THREADS, 0);
+    if (rows) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_geometry_rows<true, true>, GEO_THREADS, 0);
     else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_geometry_linear<true>, GEO_THREADS, 0);
     return n > 0 ? n : 1;
 }
@@ -2629,8 +2629,8 @@ cudaError_t launch_geometry_static(const FrameConst& c, float* F, uint8_t* W, co
     const bool rows = c.footprint_holds && c.ng[0] % 4 == 0 && ((uintptr_t)F & 15u) == 0 && ((uintptr_t)W & 3u) == 0;
     const bool aligned = rows && c.ng[0] % BRICK == 0 && c.ng[1] % BRICK == 0 && c.ng[2] % BRICK == 0;
     void (*k)(FrameConst, float*, uint8_t*, const uint16_t*, Counters*, const uint32_t*) =
-        rows ? (aligned ? (c.kd_pinhole ? k_geometry_rows<true, true, true> : k_geometry_rows<false, true, true>)
-                        : (c.kd_pinhole ? k_geometry_rows<true, true, false> : k_geometry_rows<false, true, false>))
+        rows ? (aligned ? (c.kd_pinhole ? k_geometry_rows<true, true> : k_geometry_rows<false, true>)
+                        : (c.kd_pinhole ? k_geometry_rows<true, false> : k_geometry_rows<false, false>))
              : (c.kd_pinhole ? k_geometry_linear<true> : k_geometry_linear<false>);
     return launch_chained(k, dim3(rows ? grid_rows : grid_linear), dim3(GEO_THREADS), 0, stream, c, F, W, depth, ctr, geo_list);
 }

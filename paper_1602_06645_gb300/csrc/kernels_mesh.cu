@@ -473,8 +473,8 @@ __device__ __forceinline__ uint32_t texel_colour(const ColourConst& c, const uin
         wgt[a][1] = f;
         i0[a] = i;
     }
-    // the lower corner's offset, and the steps to the upper one (into the next
-    // brick from local 7; from -1, to local 0 of the first: a step of 1)
+    // the lower corner's offset, and the steps to the upper one (from local 7
+    // into the next brick, which also takes -1, local 7 of brick -1, to 0)
     const int lx = i0[0] & 7, ly = i0[1] & 7, lz = i0[2] & 7;
     const int64_t base = (((int64_t)(i0[2] >> 3) * c.ncb[1] + (i0[1] >> 3)) * c.ncb[0] + (i0[0] >> 3)) * BRICK_VOX +
                          (lz * BRICK + ly) * BRICK + lx;
