@@ -535,9 +535,12 @@ constexpr int BRICK_THREADS = 64;  // small blocks: they fit beside the band ker
 // a chain of latencies on the way to the frame's geometry update (128^3 voxels,
 // 4,096 bricks: 16.7 -> 5.5 us; 250 x 243 x 229, 29,000 bricks: 15.4 -> 8.1
 // us).  Beyond, a thread per brick, which issues a third of the instructions
-// per brick: at 512^3, 262,144 bricks, it takes 17.8 us beside the previous
-// frame's colour kernels, which the other form's instructions would hold up.
-constexpr uint32_t SMALL_BRICKS = 65536;
+// per brick and holds up less of what runs beside it.  Whole frames at 640x480,
+// eight lanes against a thread: 29.0 and 32.5 us at 15,625 bricks, 35.0 and
+// 35.6 at 32,768, 39.9 and 38.7 at 46,656, 46.6 and 44.0 at 64,000, 115 and
+// 90.5 at 262,144; calls on caller-owned volumes 20.3 and 25.5, 29.4 and 30.0,
+// 38.6 and 35.8, 48.9 and 44.9, 160 and 138.5: the line lies where they meet.
+constexpr uint32_t SMALL_BRICKS = 32768;
 template <bool SMALL>
 __global__ void __launch_bounds__(BRICK_THREADS) k_bricks(FrameConst c, const BrickSummary* __restrict__ summ,
                                                 const uint32_t* __restrict__ tiles, Counters* __restrict__ ctr,

@@ -1,7 +1,8 @@
 """The caller-owned geometry volume (tsdf_integrate_geometry_static) against
 the oracle where its kernels differ: values that overflow, a volume far from
 the world's origin (and the handle's frames there), a depth camera that is no
-pinhole (and the handle's frames with one), stream capture."""
+pinhole (and the handle's frames with one), both forms of the culling on either
+side of the line between them, stream capture."""
 import numpy as np
 import pytest
 
@@ -139,6 +140,24 @@ def test_depth_camera_that_is_no_pinhole(dims, form):
     Kd = np.array(SKEWED[form], np.float32)
     F0, W0 = zeros(dims)
     assert check(dims, s, F0, W0, [surface(k) for k in range(3)], Kd, POSES) > F0.size // 20
+
+
+@pytest.mark.parametrize("dims", [(256, 256, 256), (256, 256, 264), (253, 250, 264)])
+def test_culling_on_both_sides_of_the_eight_lane_form(dims):
+    """32,768 bricks (the last of the eight-lane form) and 33,792, in whole bricks and ragged ones."""
+    s = float(np.float32(1.0 / 264))
+    seq = synth.sequence_small(n_frames=2, seed=11)
+    F0, W0 = zeros(dims)
+    frames = [seq.frame(k)[0] for k in range(2)]
+    assert check(dims, s, F0, W0, frames, seq.K_depth, seq.poses) > 10000
+    outs = []
+    for culling in (True, False):
+        with T.Volume(dims, dims, s, 3 * s, 64, culling=culling) as v:
+            for k in range(2):
+                v.integrate(*seq.frame(k), seq.K_depth, seq.K_rgb, seq.poses[k], seq.T_depth_rgb)
+            outs.append(v.read())
+    for a, b in zip(*outs):
+        np.testing.assert_array_equal(a, b)
 
 
 def test_captured_calls():
