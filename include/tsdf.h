@@ -352,7 +352,8 @@ tsdf_status tsdf_batch_synchronize(tsdf_batch* batch);
 /* The schedule of the batched step: blocks per SM of the persistent grid
  * (1..max_blocks_per_sm), listed bricks per work item of the geometry and
  * band phases (1..TSDF_BATCH_MAX_BRICKS_PER_ITEM: a warp takes that many
- * consecutive bricks of one scan's list at a time) and whether the step runs
+ * consecutive bricks of one scan's list at a time, the geometry phase at
+ * least two) and whether the step runs
  * as a CUDA graph.  Results do not depend on the schedule. */
 #define TSDF_BATCH_MAX_BRICKS_PER_ITEM 8
 tsdf_status tsdf_batch_set_schedule(tsdf_batch* batch, int32_t blocks_per_sm, int32_t bricks_per_item,

@@ -2358,8 +2358,10 @@ __global__ void __launch_bounds__(COL_THREADS, 4) k_batch_step(const ScanDesc* _
     // P2: geometry, one warp per item of consecutive listed bricks of a scan.
     // A warp's counts go to a scan's counters when it leaves the scan (an
     // atomic per item, tens of thousands on one address, took up to two thirds
-    // of this phase).  At least two consecutive bricks per item here: with single ones the phase
-    // takes 93-128 us for 12 scans of edges 80-328, with pairs 68-87.
+    // of this phase).  At least two consecutive bricks per item here, whatever
+    // the schedule says: with single ones the phase takes 93-128 us for 12
+    // scans of edges 80-328, with pairs 68-87 (schedules of one and two bricks
+    // per item differ in the band phase only).
     const uint32_t gtile = max(tile, 2);
     scan_prefix(pre, n, 1, [&](int i) {
         return (descs[i].scr.ctr->n_geo + descs[i].scr.ctr->n_geo_open + gtile - 1) / gtile;
@@ -2398,7 +2400,8 @@ __global__ void __launch_bounds__(COL_THREADS, 4) k_batch_step(const ScanDesc* _
             const DepthMm dm{d.depth};
             // the usual camera and mode: without the per-voxel image tests for
             // bricks inside the image and without bounds tests for whole-brick
-            // volumes; the general form handles every other brick
+            // volumes, and by weights alone for open bricks; the general form
+            // handles every other brick (those of ragged volumes, open or not)
             if (d.c.kd_pinhole && d.c.free_space && aligned)
                 geometry_item<true, true, true>(d.c, d.vol, dm, e, open, at, lane, count, changed);
             else if (d.c.kd_pinhole && d.c.free_space)
