@@ -21,11 +21,12 @@
 // read (about 130 instructions each), then the hit's six gradient samples,
 // which the lanes of a warp finish together after the march (inside it, lanes
 // that hit at different samples had run them one after another).
-// Measured (24 frames around a scene of 20 primitives, 2 m cube): 640x480 rays
-// through 512^3, 1064 -> 256 us and 5 us for the map; 1920x1080 through 192^3,
-// 1936 -> 689 us and 3 us; the three prediction levels of a tracked frame at
-// 512^3, 2454 -> 613 us one after another, about 430 us beside one another
-// (launch_raycast, RayLink).  Eight blocks per SM; 7, 10 and 12 were slower.
+// Measured, the kernel alone, on one scene (24 frames around 20 primitives in
+// a 2 m cube): 640x480 rays through 512^3, 1064 -> 256 us and 5.6 us for the map;
+// 1920x1080 through 192^3, 1936 -> 703 us and 3 us; on another scene 341 and
+// 960 us.  The three prediction levels of a tracked frame at 512^3, 2454 -> 613
+// us one after another, about 430 us beside one another (launch_raycast,
+// RayLink).  Eight blocks per SM; 7, 10 and 12 were slower.
 #include <cfloat>
 #include <cstdint>
 
@@ -232,9 +233,9 @@ __device__ __forceinline__ bool rc_pair(const RayConst& c, const float* __restri
 // filling the SMs this one's last rays leave, and one block ends only after
 // the cast before it has, so the last cast's end is the end of all.  A cast
 // by itself runs without these, which held eight bytes more per thread
-// (spilled): 640x480 through 512^3 328 -> 310 us, 1920x1080 through 192^3
-// 883 -> 789 us; three chained casts 25 us less with one waiting thread
-// instead of all.
+// (spilled): whole calls, over several scenes, 640x480 through 512^3 328 -> 310
+// us, 1920x1080 through 192^3 883 -> 789 us; three chained casts 25 us less
+// with one waiting thread instead of all.
 template <bool CHAIN>
 __global__ void __launch_bounds__(RC_THREADS, 8) k_raycast(RayConst c, const float* __restrict__ F,
                                                         const uint8_t* __restrict__ W, const uint32_t* __restrict__ C,
