@@ -20,16 +20,26 @@ namespace {
 // per thread and 64-bit divisions for its coordinates they took 4.3 ms and
 // 0.48 ms.  A 750 x 729 x 687 colour volume (8-byte accesses) runs at 6.4
 // (read-out) and 7.0 TB/s (restore), 1.36 ms each way before, 0.23-0.25 now.
-template <typename V, int VE, bool TO_LINEAR>
+// NARROW (rows of at most one brick, 8 voxels): at most 8 lanes along x and the
+// rest along y, where the wide form leaves 31 of 32 lanes idle at nx = 1.  The
+// three volumes of a call read out: 1 x 512 x 512 46 -> 33 us, 3 x 700 x 700 60 ->
+// 45, 8 x 1024 x 1024 83 -> 70.
+template <int VE, bool NARROW>
+struct ConvertShape {
+    static constexpr int XL = NARROW ? (VE == 1 ? 8 : 4) : 32 / VE, YL = 32 / XL;  // lanes along x and y
+    static constexpr int XW = XL * VE;                                             // voxels of a chunk along x
+    static constexpr int XC = NARROW ? 1 : (VE == 8 ? 4 : (VE == 4 ? 2 : 1));      // chunks per warp
+    static constexpr int YI = BRICK / YL;                                          // row steps
+};
+template <typename V, int VE, bool NARROW, bool TO_LINEAR>
 __global__ void __launch_bounds__(256) k_convert(V* __restrict__ brick, V* __restrict__ lin, int nx, int ny, int nz,
                                                  int z0, int nbx, int nby) {
-    constexpr int XL = 32 / VE;                           // lanes along x; VE lanes along y
-    constexpr int XC = VE == 8 ? 4 : (VE == 4 ? 2 : 1);   // 32-voxel chunks per warp
-    constexpr int YI = BRICK / VE;                        // row steps
+    using S = ConvertShape<VE, NARROW>;
+    constexpr int XL = S::XL, YL = S::YL, XW = S::XW, XC = S::XC, YI = S::YI;
     const int lane = threadIdx.x & 31, z = blockIdx.z * BRICK + (threadIdx.x >> 5);
     if (z >= nz) return;
     const int by = blockIdx.y, ly = lane / XL, gz = z0 + z;
-    const int x0 = blockIdx.x * (32 * XC) + (lane % XL) * VE;
+    const int x0 = blockIdx.x * (XW * XC) + (lane % XL) * VE;
     const int64_t brow = (((int64_t)(gz >> 3) * nby + by) * nbx) * BRICK_VOX + (gz & 7) * (BRICK * BRICK);
     const int64_t lrow = ((int64_t)z * ny + by * BRICK) * nx;
     V v[XC][YI];
@@ -37,7 +47,7 @@ __global__ void __launch_bounds__(256) k_convert(V* __restrict__ brick, V* __res
     for (int c = 0; c < XC; ++c)
 #pragma unroll
         for (int r = 0; r < YI; ++r) {
-            const int x = x0 + 32 * c, y = ly + VE * r;
+            const int x = x0 + XW * c, y = ly + YL * r;
             if (x < nx && by * BRICK + y < ny)
                 v[c][r] = TO_LINEAR ? brick[(brow + (int64_t)(x >> 3) * BRICK_VOX + y * BRICK + (x & 7)) / VE]
                                     : lin[(lrow + (int64_t)y * nx + x) / VE];
@@ -46,7 +56,7 @@ __global__ void __launch_bounds__(256) k_convert(V* __restrict__ brick, V* __res
     for (int c = 0; c < XC; ++c)
 #pragma unroll
         for (int r = 0; r < YI; ++r) {
-            const int x = x0 + 32 * c, y = ly + VE * r;
+            const int x = x0 + XW * c, y = ly + YL * r;
             if (x < nx && by * BRICK + y < ny) {
                 if (TO_LINEAR)
                     lin[(lrow + (int64_t)y * nx + x) / VE] = v[c][r];
@@ -56,15 +66,20 @@ __global__ void __launch_bounds__(256) k_convert(V* __restrict__ brick, V* __res
         }
 }
 
+template <typename V, int VE, bool NARROW, bool TO_LINEAR>
+cudaError_t convert_grid(void* brick, void* lin, const int32_t dims[3], int z0, int z1, cudaStream_t stream) {
+    constexpr int XW = ConvertShape<VE, NARROW>::XW * ConvertShape<VE, NARROW>::XC;  // voxels of a warp
+    const int nbx = (dims[0] + BRICK - 1) / BRICK, nby = (dims[1] + BRICK - 1) / BRICK;
+    const dim3 grid((unsigned)((dims[0] + XW - 1) / XW), (unsigned)nby, (unsigned)((z1 - z0 + BRICK - 1) / BRICK));
+    k_convert<V, VE, NARROW, TO_LINEAR><<<grid, 256, 0, stream>>>(static_cast<V*>(brick), static_cast<V*>(lin), dims[0],
+                                                                  dims[1], z1 - z0, z0, nbx, nby);
+    return cudaGetLastError();
+}
+
 template <typename V, int VE, bool TO_LINEAR>
 cudaError_t convert_as(void* brick, void* lin, const int32_t dims[3], int z0, int z1, cudaStream_t stream) {
-    constexpr int XC = VE == 8 ? 4 : (VE == 4 ? 2 : 1);
-    const int nbx = (dims[0] + BRICK - 1) / BRICK, nby = (dims[1] + BRICK - 1) / BRICK;
-    const dim3 grid((unsigned)((dims[0] + 32 * XC - 1) / (32 * XC)), (unsigned)nby,
-                    (unsigned)((z1 - z0 + BRICK - 1) / BRICK));
-    k_convert<V, VE, TO_LINEAR><<<grid, 256, 0, stream>>>(static_cast<V*>(brick), static_cast<V*>(lin), dims[0],
-                                                          dims[1], z1 - z0, z0, nbx, nby);
-    return cudaGetLastError();
+    return dims[0] <= BRICK ? convert_grid<V, VE, true, TO_LINEAR>(brick, lin, dims, z0, z1, stream)
+                            : convert_grid<V, VE, false, TO_LINEAR>(brick, lin, dims, z0, z1, stream);
 }
 
 // The widest access whose size divides both base addresses and the linear row
