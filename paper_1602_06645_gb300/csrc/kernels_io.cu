@@ -99,14 +99,16 @@ cudaError_t convert(T* brick, T* lin, const int32_t dims[3], int z0, int z1, cud
     return convert_as<uint8_t, 1, TO_LINEAR>(brick, lin, dims, z0, z1, stream);
 }
 
-// Brick summaries: min/max of F over observed voxels, min of w over in-volume
-// voxels (never max_weight where some w lies above it) and the band flags
-// (what the geometry kernel maintains).  Bound by HBM (5 B per voxel).  One
-// warp per brick with the geometry kernel's lane layout (lane l: voxels
-// 4 (l + 32 j) .. + 3, j = 0..3), all eight 16- and 4-byte reads of a lane
-// issued together; the flags come from the minima and maxima over the lane's
-// faces: 118 us at 512^3 (5.7 TB/s); one block per brick with scalar reads and
-// a shared-memory reduction took 235 us.
+// Brick summaries: min/max of F over observed voxels, whether all of them are
+// observed and at the weight limit (wmin) and the band flags (what the
+// geometry kernel maintains).  Bound by HBM (5 B per voxel).  One warp per
+// brick with the geometry kernel's lane layout (lane l: voxels 4 (l + 32 j) ..
+// + 3, j = 0..3), all eight 16- and 4-byte reads of a lane issued together; the
+// flags come from the minima and maxima over the lane's faces, the weights are
+// tested four at a time.  About 103 us at 512^3 (6.5 TB/s; 118 with a minimum
+// per weight, 128 with a test for weights above the limit beside it, whose 40
+// registers leave 48 warps per SM instead of 64); one block per brick with
+// scalar reads and a shared-memory reduction took 235 us.
 constexpr int SUM_WARPS = 8;
 __global__ void __launch_bounds__(SUM_WARPS * 32) k_summaries(const float* __restrict__ F,
                                                               const uint8_t* __restrict__ W,
@@ -128,21 +130,25 @@ __global__ void __launch_bounds__(SUM_WARPS * 32) k_summaries(const float* __res
     }
     const float inf = __int_as_float(0x7f800000), qnan = __int_as_float(0x7fffffff);
     float mn = inf, mx = -inf, mn_xf = inf, mx_xf = -inf, mn_zf = inf, mx_zf = -inf;
-    uint32_t wmn = 0xFFFFFFFFu, wmx = 0u;
+    const uint32_t limit4 = max_weight * 0x01010101u;
+    uint32_t xin = 0u;  // this lane's bytes inside the volume along x
+#pragma unroll
+    for (int i = 0; i < 4; ++i) xin |= bx * BRICK + lx + i < nx ? 0xFFu << (8 * i) : 0u;
+    uint32_t hole = 0u, differs = 0u;  // an unobserved voxel (bit 7 of some byte); a weight that is not the limit
     bool odd = false;
+    // (voxels outside the volume hold F = 0 and w = 0)
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         const bool in = by * BRICK + ly < ny && bz * BRICK + lz + 2 * j < nz;
         const float fv[4] = {f[j].x, f[j].y, f[j].z, f[j].w};
+        const uint32_t inside = in ? xin : 0u, wq = (w[j] & inside) | (limit4 & ~inside);
+        hole |= (wq - 0x01010101u) & ~wq;
+        differs |= wq ^ limit4;
         float gmn = inf, gmx = -inf;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const bool vox = in && bx * BRICK + lx + i < nx;
-            const uint32_t wi = (w[j] >> (8 * i)) & 0xFFu;
-            wmn = min(wmn, vox ? wi : 0xFFFFFFFFu);
-            wmx = max(wmx, vox ? wi : 0u);
-            odd = odd || (vox && !(fabsf(fv[i]) <= PLAIN_F));
-            const float v = vox && wi ? fv[i] : qnan;  // fminf / fmaxf pass over a NaN
+            odd = odd || !(fabsf(fv[i]) <= PLAIN_F);
+            const float v = (w[j] >> (8 * i)) & 0xFFu ? fv[i] : qnan;  // fminf / fmaxf pass over a NaN
             gmn = fminf(gmn, v);
             gmx = fmaxf(gmx, v);
             if (i == (lx ? 3 : 0)) {  // the lane's x-face voxel
@@ -164,10 +170,10 @@ __global__ void __launch_bounds__(SUM_WARPS * 32) k_summaries(const float* __res
                      (lz == 0 ? zf << 10 : zf << 12);
     if (__any_sync(0xffffffffu, odd) && lane == 0) *odd_f = 1u;
     flags = __reduce_or_sync(0xffffffffu, flags);
-    wmn = __reduce_min_sync(0xffffffffu, wmn);
-    // a weight above the limit comes down to it at its next update: the brick
-    // is not saturated, which wmin == max_weight would say
-    if (__reduce_max_sync(0xffffffffu, wmx) > max_weight && wmn == max_weight) ++wmn;
+    // (a weight above the limit comes down to it at its next update: the brick
+    // is not saturated)
+    const bool unobserved = __any_sync(0xffffffffu, (hole & 0x80808080u) != 0u);
+    const bool below_cap = __any_sync(0xffffffffu, differs != 0u);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
@@ -177,7 +183,7 @@ __global__ void __launch_bounds__(SUM_WARPS * 32) k_summaries(const float* __res
         BrickSummary s;
         s.fmin = mn >= FLT_MAX ? inf : mn;
         s.fmax = mx <= -FLT_MAX ? -inf : mx;
-        s.wmin = wmn == 0xFFFFFFFFu ? 0u : wmn;
+        s.wmin = unobserved ? 0u : (below_cap ? max_weight - 1u : max_weight);
         s.flags = flags;
         summ[b] = s;
     }
