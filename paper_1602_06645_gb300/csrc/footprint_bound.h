@@ -48,6 +48,7 @@ inline bool footprint_holds(const float R[9], const float t[3], const float K[9]
         double g = 0.0;
         for (int q = 0; q < 3; ++q)
             for (int a = 0; a < 3; ++a) g += std::fabs((double)Kinv[3 * r + a] * (double)K[3 * a + q]);
+        if (!(g < 1e9)) return false;  // (an inverse that overflows binary32 makes it infinite or not a number)
         G = std::max(G, g);
     }
     // the reciprocal of K's third row times a camera point is exact between 2^-126 and 2^126

@@ -24,6 +24,15 @@ int main(int argc, char** argv) {
     std::mt19937_64 rng(7);
     auto uni = [&](double lo, double hi) { return std::uniform_real_distribution<double>(lo, hi)(rng); };
     auto logu = [&](double lo, double hi) { return std::pow(10.0, uni(std::log10(lo), std::log10(hi))); };
+    {  // intrinsics whose inverse overflows, a camera at infinity, voxels of no size
+        const float I[9] = {1, 0, 0, 0, 1, 0, 0, 0, 1}, o[3] = {0, 0, 0}, t[3] = {0, 0, 2}, far[3] = {0, 0, INFINITY};
+        const float K[9] = {500, 0, 320, 0, 500, 240, 0, 0, 1}, Ki[9] = {0.002f, 0, -0.64f, 0, 0.002f, -0.48f, 0, 0, 1};
+        const float Kz[9] = {1e-39f, 0, 320, 0, 500, 240, 0, 0, 1}, Kzi[9] = {INFINITY, 0, -INFINITY, 0, 0.002f, -0.48f, 0, 0, 1};
+        const int32_t nb[3] = {8, 8, 8};
+        if (!tsdf::footprint_holds(I, t, K, Ki, o, nb, 0, 0.01f) || tsdf::footprint_holds(I, t, Kz, Kzi, o, nb, 0, 0.01f) ||
+            tsdf::footprint_holds(I, far, K, Ki, o, nb, 0, 0.01f) || tsdf::footprint_holds(I, t, K, Ki, o, nb, 0, 1e-9f))
+            return 2;
+    }
     long inner_holds = 0, inner_not = 0, wrong_holds = 0, wrong_not = 0, near_not = 0, near = 0;
     for (int n = 0; n < samples; ++n) {
         Camera c{};
